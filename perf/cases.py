@@ -365,3 +365,69 @@ def tolerance(case):
     # have is the distance to the ordered mode, where no item sees another's update; measured at the listed sizes: 1.2e-5
     # (largest single value 0.017), 5e-4 (0.038: the first AdaGrad steps are long whatever the gradient), 7e-5 (1e-4).
     return {"sgns": {"rel": 5e-5, "max": 0.07}, "complex": {"rel": 1.5e-3, "max": 0.15}, "mf": {"rel": 3e-4, "max": 1e-3}}[k]
+
+
+# ------------------------------------------------------------------------------------------------
+# the same results in 64 bits, without the framework
+# ------------------------------------------------------------------------------------------------
+def _start_values(keys, length, seed, which, scale):
+    """The start values of a table (uniform in [-scale, scale)), from the published generator: Philox4x32-10 with the counter
+    (block of four values, table, 3) and the seed as its key; 24 bits of a word make a value."""
+    out = torch.empty(keys * length, dtype=torch.float64, device="cuda")
+    unit = float(np.float32(scale) * np.float32(1.0 / 8388608.0))
+    low, step = 0xFFFFFFFF, 1 << 26
+
+    def product(a, b):                                      # high and low half of a 32 x 32-bit product, in 64-bit integers
+        lo = a * (b & 0xFFFF)
+        hi = a * (b >> 16) + (lo >> 16)
+        return hi >> 16, ((hi & 0xFFFF) << 16) | (lo & 0xFFFF)
+
+    for first in range(0, out.numel() // 4, step):
+        i = torch.arange(first, min(first + step, out.numel() // 4), device="cuda")
+        c = [i & low, i >> 32, torch.full_like(i, which), torch.full_like(i, 3)]
+        k0, k1 = seed & low, (seed >> 32) & low
+        for _ in range(10):
+            h0, l0 = product(c[0], 0xD2511F53)
+            h1, l1 = product(c[2], 0xCD9E8D57)
+            c = [h1 ^ c[1] ^ k0, l1, h0 ^ c[3] ^ k1, l0]
+            k0, k1 = (k0 + 0x9E3779B9) & low, (k1 + 0xBB67AE85) & low
+        words = torch.stack([(w >> 8) - 8388608 for w in c], dim=1).to(torch.float32) * unit     # rounded as the table holds it
+        out[4 * first:4 * first + words.numel()] = words.reshape(-1).double()
+    return out.view(keys, length)
+
+
+def _keys_of(keys, n, skew, seed):
+    """The first key batch of a state."""
+    return inputs.zipf_keys(n, keys, skew, seed * BATCHES, "cuda", cdf=inputs.zipf_cdf(keys, skew, "cuda") if skew else None).long()
+
+
+def exact(case, seed):
+    """What the first pass returns, in 64 bits.  None: copies and whole numbers; steps in which items race, where any order of
+    them is right; steps whose negatives come from the store's own sampler."""
+    c, seed = case, int(seed)
+    if c["kind"] == "push":
+        table = _start_values(c["keys"], c["len"], seed, 0, 0.1)
+        dtype = torch.float64 if c["bytes"] == 8 else torch.float32
+        delta = torch.randn((c["n"], c["len"]), generator=_gen(seed, 1), device="cuda", dtype=dtype)
+        return table.index_add_(0, _keys_of(c["keys"], c["n"], c["skew"], seed), delta.double())
+    if c["kind"] == "round":
+        tables = _start_values(c["keys"], c["len"], seed, 0, 0.1), _start_values(c["keys"], c["len"], seed + 1, 1, 0.1)
+        keys = _keys_of(c["keys"], c["n"], c["skew"], seed)
+        dtype = torch.float64 if c["bytes"] == 8 else torch.float32
+        delta = torch.randn((c["n"], c["len"]), generator=_gen(seed, 1), device="cuda", dtype=dtype)
+        pulled = tables[0][keys], tables[1][keys]
+        tables[0].index_add_(0, keys, delta.double())
+        tables[1].index_add_(0, keys, (delta ** 2).double())
+        return (*pulled, tables)
+    if c["kind"] == "mf" and c["ordered"]:
+        M, N, B = c["rows"], c["cols"], c["batch"]
+        table = _start_values(M + N, c["len"], seed, 0, 0.3)
+        i, j, x = inputs.mf_cells(BATCHES * B, M, N, 0.8, c["len"], 0.1, seed, "cuda", by_column_of=100 * M if c["columns"] else 0)
+        i, j, x = i[:B].long(), j[:B].long(), x[:B].double()
+        rate, decay = float(np.float32(1e-4)), float(np.float32(0.01))
+        w, h = table[i], table[j]
+        err = x - (w * h).sum(1)
+        table.index_add_(0, i, rate * (err[:, None] * h - decay * w))
+        table.index_add_(0, j, rate * (err[:, None] * w - decay * h))
+        return (err ** 2).mean().reshape(1), table
+    return None
