@@ -1045,15 +1045,19 @@ __global__ void clip_fold_kernel(DevStat* st, const float2* __restrict__ clip_it
 }
 
 // mean of the per-item losses, summed in a fixed order
-__global__ void loss_mean_kernel(const float* __restrict__ loss_item, uint64_t n, float* __restrict__ out)
+constexpr unsigned LOSS_THREADS = 1024;
+__global__ void __launch_bounds__(LOSS_THREADS)
+loss_mean_kernel(const float* __restrict__ loss_item, uint64_t n, float* __restrict__ out)
 {
-    __shared__ double sh[256];
+    grid_dependency_wait();
+    __shared__ double sh[LOSS_THREADS];
     double s = 0.0;
-    for (uint64_t i = threadIdx.x; i < n; i += 256) s += (double)loss_item[i];
+#pragma unroll 8
+    for (uint64_t i = threadIdx.x; i < n; i += LOSS_THREADS) s += (double)loss_item[i];
     sh[threadIdx.x] = s;
     __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if ((int)threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
+    for (unsigned o = LOSS_THREADS / 2; o > 0; o >>= 1) {
+        if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
         __syncthreads();
     }
     if (threadIdx.x == 0) *out = (float)(sh[0] / (double)(n ? n : 1));
@@ -1106,7 +1110,7 @@ static nups_status step_finish(nups_store* s, uint64_t n, uint64_t per, const St
         if (rc != NUPS_OK) return rc;
     }
     if (d_loss_out && !loss_done_in_kernel) {
-        loss_mean_kernel<<<1, 256, 0, st>>>(b.loss_item, n, d_loss_out);
+        nups_launch_dependent(loss_mean_kernel, 1, LOSS_THREADS, 0, st, b.loss_item, n, d_loss_out);
         LAUNCH_CHECK(s);
     }
     if (clips && s->cfg.clip_factor > 0.f && s->H) {

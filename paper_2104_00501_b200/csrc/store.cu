@@ -4,7 +4,10 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <type_traits>
+
 #include "nups_internal.cuh"
+#include "nups_sort.cuh"
 
 thread_local char g_nups_cuda_err[256] = "";
 
@@ -848,93 +851,372 @@ push_atomic_kernel(View v, const uint32_t* __restrict__ keys, uint64_t n, PushPa
 }
 
 // ---------------------------------------------------------------------------------------------
-// push, deterministic mode: rows are sorted (stably) by destination, then one warp per
-// destination adds its rows one by one in input order.
+// push, deterministic mode: the rows of one destination are added one by one in input order.  A destination is one
+// number: the key, or num_keys + worker * H + slot for a replica row; num_keys + R * H marks a bad key.
+// Measured: 200,003 rows of 64 floats (Zipf 0.9 over 2M keys, 1,000 of them replicated) 430 -> 96 us with the merge: keys
+// 14, three sort passes 36, push_apply_kernel 28, push_chain_kernel 10 us.
+//   n <= SMALL_PUSH_ROWS: one launch without any sorting (push_small_kernel).
+//   else: the rows are sorted stably by destination (nups_sort.cuh), push_apply_kernel adds the rows of every destination
+//   that has at most APPLY_ROWS of them, and push_chain_kernel those of the few that have more.
 // ---------------------------------------------------------------------------------------------
-template <bool HOT>
-__global__ void push_dest_kernel(View v, const uint32_t* __restrict__ keys, uint64_t n, uint64_t n_items,
-                                 uint32_t rows_per_item, unsigned long long invalid_dest,
-                                 unsigned long long* __restrict__ dest, uint32_t* __restrict__ idx)
-{
-    uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const unsigned lane = threadIdx.x & 31;
-    bool in = i < n;
-    uint32_t key = in ? keys[i] : 0u;
-    bool valid = in && key < v.num_keys;
-    if (in && !valid) flag_bad_key(v);
-    bool hot = false;
-    unsigned long long d = invalid_dest;
-    if (valid) {
-        d = key;
-        if (HOT && key_is_hot(v, key)) {
-            hot = true;
-            uint32_t slot = (uint32_t)v.slot_of[key];
-            uint32_t q = worker_of_item(i / rows_per_item, n_items, v.R);
-            d = (1ull << 32) + (unsigned long long)q * v.H + slot;
-            if (v.dirty[(size_t)q * v.Hcap + slot] == 0u) v.dirty[(size_t)q * v.Hcap + slot] = 1u;
+template <class K, bool HOT>
+struct PushDest {
+    View v;
+    const uint32_t* keys;
+    uint64_t n_items;
+    uint32_t rows_per_item;
+    bool note;                  // count the accesses, flag bad keys, mark the replicas as touched
+
+    __device__ __forceinline__ K invalid() const { return (K)v.num_keys + (K)((uint64_t)v.R * v.H); }
+    // rows i, i + step, ...; called by whole warps.  The lookups of the rows go side by side: each is a chain of up to three
+    // dependent loads.
+    template <int N>
+    __device__ __forceinline__ void operator()(uint64_t i, uint64_t step, uint64_t n, K (&d)[N]) const
+    {
+        uint32_t key[N], bits[N], slot[N];
+#pragma unroll
+        for (int m = 0; m < N; ++m) key[m] = i + m * step < n ? __ldg(keys + i + m * step) : 0u;
+#pragma unroll
+        for (int m = 0; m < N; ++m) bits[m] = HOT && key[m] < v.num_keys ? __ldg(v.hot_bits + (key[m] >> 5)) >> (key[m] & 31) & 1u : 0u;
+#pragma unroll
+        for (int m = 0; m < N; ++m) slot[m] = HOT && bits[m] ? (uint32_t)__ldg(v.slot_of + key[m]) : 0u;
+        uint32_t* flag[N];
+        bool clean[N];
+#pragma unroll
+        for (int m = 0; m < N; ++m) {
+            const uint64_t row = i + m * step;
+            const bool valid = row < n && key[m] < v.num_keys;
+            d[m] = valid ? (K)key[m] : invalid();
+            flag[m] = nullptr;
+            if (HOT && valid && bits[m]) {
+                const uint32_t q = worker_of_item(rows_per_item == 1 ? row : row / rows_per_item, n_items, v.R);
+                d[m] = (K)v.num_keys + (K)((uint64_t)q * v.H + slot[m]);
+                flag[m] = v.dirty + (size_t)q * v.Hcap + slot[m];
+            }
+            clean[m] = note && flag[m] && *flag[m] == 0u;
+        }
+#pragma unroll
+        for (int m = 0; m < N; ++m) {
+            const bool in = i + m * step < n, valid = in && key[m] < v.num_keys, hot = flag[m] != nullptr;
+            if (clean[m]) *flag[m] = 1u;
+            if (note && in && !valid) flag_bad_key(v);
+            if (note && v.count) {
+                if (valid) atomicAdd(v.cnt + key[m], 1ull);
+                const unsigned hot_m = __ballot_sync(0xFFFFFFFFu, hot);
+                const unsigned cold_m = __ballot_sync(0xFFFFFFFFu, valid && !hot);
+                if ((threadIdx.x & 31) == 0) {
+                    if (hot_m) atomicAdd(&v.st->hot_hits, (unsigned long long)__popc(hot_m));
+                    if (cold_m) atomicAdd(&v.st->cold_hits, (unsigned long long)__popc(cold_m));
+                }
+            }
         }
     }
-    if (in) { dest[i] = d; idx[i] = (uint32_t)i; }
-    if (v.count) {
-        if (valid) atomicAdd(v.cnt + key, 1ull);
-        unsigned hot_m = __ballot_sync(0xFFFFFFFFu, valid && hot);
-        unsigned cold_m = __ballot_sync(0xFFFFFFFFu, valid && !hot);
-        if (lane == 0) {
-            if (hot_m) atomicAdd(&v.st->hot_hits, (unsigned long long)__popc(hot_m));
-            if (cold_m) atomicAdd(&v.st->cold_hits, (unsigned long long)__popc(cold_m));
+};
+
+// first 16-byte chunk of a destination's row in the value (which = 0) or accumulator table
+template <class K>
+__device__ __forceinline__ float4* dest_row(const View& v, K d, int which)
+{
+    if (d < (K)v.num_keys) return (float4*)(which ? v.acc : v.val) + (uint64_t)d * v.L4;
+    const K r = d - (K)v.num_keys, q = r / (K)v.H, slot = r - q * (K)v.H;
+    return (float4*)(which ? v.dacc : v.dval) + ((uint64_t)q * v.Hcap + slot) * v.L4;
+}
+
+constexpr uint32_t APPLY_ROWS = 32;          // destinations with more rows than this go to push_chain_kernel
+constexpr unsigned APPLY_THREADS = 256;
+
+// A warp takes the destinations that begin in its window of sorted positions.  W lanes serve one destination (rows of up to
+// 16 chunks leave half a warp or more idle otherwise), each group of lanes works on two destinations at a time: most
+// destinations have one or two rows, so what counts is how many row fetches are outstanding.  The window is short enough
+// that a group of lanes has at most four such pairs to take one after the other.  (Lanes of their own for every position,
+// whether a destination begins there or not, hide latency better but take 2.5 times the instructions: 54 us instead of
+// 37 us for 200,000 rows of 64 floats.)
+template <int W> constexpr unsigned APPLY_WINDOW = 4 * 2 * 32 / W;
+
+template <class K, bool F64, int W>
+__global__ void __launch_bounds__(APPLY_THREADS, 4)
+push_apply_kernel(View v, const K* __restrict__ dest, const uint32_t* __restrict__ idx, uint64_t n64, K invalid,
+                  const float4* __restrict__ dv, const float4* __restrict__ da, uint32_t* __restrict__ longs,
+                  uint32_t* __restrict__ long_count)
+{
+    grid_dependency_wait();
+    constexpr unsigned FULL = 0xFFFFFFFFu;
+    constexpr int GROUPS = 32 / W, U = 2;
+    constexpr unsigned WIN = APPLY_WINDOW<W>;
+    static_assert(WIN <= 32, "a window is looked at by one warp");
+    __shared__ uint32_t s_idx[APPLY_THREADS / 32][WIN];
+    __shared__ K s_dest[APPLY_THREADS / 32][WIN];
+    __shared__ uint8_t s_begin[APPLY_THREADS / 32][WIN];           // where the window's destinations begin, in order
+    const unsigned lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    const uint64_t base64 = (((uint64_t)blockIdx.x * APPLY_THREADS + threadIdx.x) >> 5) * WIN;
+    if (base64 >= n64) return;
+    const uint32_t base = (uint32_t)base64, n = (uint32_t)n64;     // positions fit 32 bits; sums with a window may not
+    const bool look = lane < WIN, in = look && base64 + lane < n64;
+    const K d = in ? dest[base64 + lane] : invalid;
+    K before = __shfl_up_sync(FULL, d, 1);
+    if (lane == 0) before = base ? dest[base - 1] : d;
+    const bool begins = look && (before != d || base64 + lane == 0);
+    const unsigned bounds = __ballot_sync(FULL, begins);           // bad keys and the end of the input sort last: one run
+    const unsigned nb = __popc(bounds), nh = __popc(__ballot_sync(FULL, begins && d != invalid));
+    if (begins) s_begin[wib][__popc(bounds & ((1u << lane) - 1u))] = (uint8_t)lane;
+    if (look) { s_idx[wib][lane] = in ? idx[base64 + lane] : 0u; s_dest[wib][lane] = d; }
+    __syncwarp();
+    const unsigned group = lane / W, c0 = lane % W;
+    const uint32_t L4 = v.L4;
+    // row numbers of the destination's rows: `at` counts from the window's first position
+    auto row_at = [&](uint32_t at) -> uint64_t { return (uint64_t)(at < WIN ? s_idx[wib][at] : idx[base64 + at]) * L4; };
+    for (unsigned k0 = group; k0 < nh; k0 += U * GROUPS) {
+        uint32_t begin[U], end[U];
+        float4* row[U];
+        bool live[U];
+        K to[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const unsigned k = k0 + u * GROUPS;
+            live[u] = k < nh;
+            begin[u] = end[u] = 0;
+            to[u] = invalid;
+            if (!live[u]) continue;
+            begin[u] = s_begin[wib][k];
+            to[u] = s_dest[wib][begin[u]];
+            if (k + 1 < nb) { end[u] = s_begin[wib][k + 1]; continue; }
+            uint32_t e = WIN;
+            if (base64 + e < n64 && dest[base64 + e] == to[u]) {
+                if (base64 + begin[u] + APPLY_ROWS < n64 && dest[base64 + begin[u] + APPLY_ROWS] == to[u]) {
+                    if (c0 == 0) longs[atomicAdd(long_count, 1u)] = base + begin[u];
+                    live[u] = false;
+                } else {
+                    while (base64 + e < n64 && dest[base64 + e] == to[u]) ++e;
+                }
+            }
+            end[u] = min(e, n - base);
+        }
+#pragma unroll
+        for (int which = 0; which < 2; ++which) {
+            const float4* src = which ? da : dv;
+            if (!src) continue;
+#pragma unroll
+            for (int u = 0; u < U; ++u) row[u] = live[u] ? dest_row<K>(v, to[u], which) : nullptr;
+            for (uint32_t c = c0; c < L4; c += W) {
+                float4 a[U], x[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    if (live[u]) { a[u] = row[u][c]; x[u] = ld_stream_v4(src + row_at(begin[u]) + c); }
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    if (!live[u]) continue;
+                    a[u] = add_chunk<F64>(a[u], x[u]);
+                    for (uint32_t at = begin[u] + 1; at < end[u]; at += 4) {       // loads issued together, additions kept in order
+                        float4 y[4];
+#pragma unroll
+                        for (int m = 0; m < 4; ++m)
+                            if (at + m < end[u]) y[m] = ld_stream_v4(src + row_at(at + m) + c);
+#pragma unroll
+                        for (int m = 0; m < 4; ++m)
+                            if (at + m < end[u]) a[u] = add_chunk<F64>(a[u], y[m]);
+                    }
+                    row[u][c] = a[u];
+                }
+            }
         }
     }
 }
 
-template <bool F64>
-__global__ void __launch_bounds__(256)
-push_ordered_kernel(View v, const unsigned long long* __restrict__ dest, const uint32_t* __restrict__ idx, uint64_t n,
-                    unsigned long long invalid_dest, const float4* __restrict__ dv, const float4* __restrict__ da)
+// Destinations with many rows (a frequent key): a chain of dependent additions per value, which only the columns can
+// share out.  One block takes one group of 32 values of the row (CH chunks of 16 bytes).  Four warps bring the rows' parts
+// into a ring in shared memory by asynchronous copies, five stages ahead; lane l of the fifth adds up value l.  Fetched by
+// plain loads, four rows at a time, the chain would wait for memory at every fourth row.  Measured: 290,000 rows of 128 floats,
+// 93,000 of them of one key: 24.8 ms with plain loads, 0.65 ms (6 ns a row; the additions alone need about 2).
+constexpr unsigned CHAIN_THREADS = 160, CHAIN_STAGES = 6, CHAIN_STAGE_BYTES = 8192;
+constexpr unsigned CHAIN_SMEM = CHAIN_STAGES * CHAIN_STAGE_BYTES;  // 48 KB: four blocks per multiprocessor
+
+template <class K, bool F64>
+__global__ void __launch_bounds__(CHAIN_THREADS)
+push_chain_kernel(View v, const K* __restrict__ dest, const uint32_t* __restrict__ idx, uint64_t n,
+                  const float4* __restrict__ dv, const float4* __restrict__ da, const uint32_t* __restrict__ longs,
+                  const uint32_t* __restrict__ long_count)
 {
+    grid_dependency_wait();
+    using V = typename std::conditional<F64, double, float>::type;
+    constexpr unsigned FULL = 0xFFFFFFFFu;
+    constexpr uint32_t CH = 32 * sizeof(V) / 16;                   // chunks of a column group
+    constexpr uint32_t ROWS = CHAIN_STAGE_BYTES / (CH * 16);       // rows per stage
+    constexpr uint32_t COPIES = ROWS * CH / 128;                   // 16-byte copies per producing thread and stage
+    constexpr uint32_t LOOK = 4;                                   // stages whose row numbers are looked up at once
+    extern __shared__ __align__(16) unsigned char ring[];
     const unsigned lane = threadIdx.x & 31;
-    const uint64_t j = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (j >= n) return;
-    unsigned long long d = dest[j];
-    if (d == invalid_dest) return;
-    if (j > 0 && dest[j - 1] == d) return;           // not the first row of its destination
-    const uint32_t L4 = v.L4;
-    float4* tv;
-    float4* ta;
-    if (d >> 32) {
-        unsigned long long r = d - (1ull << 32);
-        uint64_t q = r / v.H, slot = r % v.H;
-        uint64_t off = (q * v.Hcap + slot) * L4;
-        tv = (float4*)v.dval + off;
-        ta = (float4*)v.dacc + off;
-    } else {
-        tv = (float4*)v.val + d * L4;
-        ta = (float4*)v.acc + d * L4;
+    const bool adds = threadIdx.x < 32;
+    const uint32_t L4 = v.L4, cgroups = (L4 + CH - 1) / CH, tables = (dv ? 1u : 0u) + (da ? 1u : 0u);
+    const uint64_t units = (uint64_t)*long_count * cgroups * tables;
+    const uint32_t ring_s = (uint32_t)__cvta_generic_to_shared(ring);
+    for (uint64_t unit = blockIdx.x; unit < units; unit += gridDim.x) {
+        const uint32_t cg = (uint32_t)(unit % cgroups);
+        const int which = (!dv || (unit / cgroups) % tables) ? 1 : 0;
+        const uint64_t begin = longs[unit / cgroups / tables];
+        const K d = dest[begin];
+        uint64_t lo = begin, hi = n;                               // last position known to be of d, first known not to be
+        while (hi - lo > 1) {
+            const uint64_t step = (hi - lo + 32) / 33, at = lo + (lane + 1) * step;
+            const unsigned cnt = __popc(__ballot_sync(FULL, at < hi && dest[at] == d));
+            lo += cnt * step;
+            hi = min(hi, lo + step);
+        }
+        const uint32_t rows = (uint32_t)(lo + 1 - begin), stages = (rows + ROWS - 1) / ROWS;
+        const uint32_t* my_rows = idx + begin;
+        // producing thread t copies chunk t % CH of rows t / CH, t / CH + 128 / CH, ... of a stage
+        const uint32_t t = threadIdx.x - 32, first_row = t / CH, chunk = cg * CH + t % CH;
+        const float4* src = (which ? da : dv) + chunk;
+        auto look_up = [&](uint32_t stage, uint32_t (&r)[LOOK * COPIES]) {
+#pragma unroll
+            for (uint32_t k = 0; k < LOOK * COPIES; ++k) {
+                const uint32_t row = stage * ROWS + first_row + k * (128 / CH);
+                r[k] = row < rows && chunk < L4 ? __ldg(my_rows + row) : 0xFFFFFFFFu;
+            }
+        };
+        const uint32_t col = cg * 32 + lane;                       // the value this lane adds up
+        const bool mine = adds && col < L4 * (16 / sizeof(V));
+        V* out = reinterpret_cast<V*>(dest_row<K>(v, d, which)) + col;
+        V acc = mine ? *out : V(0);
+        if (!adds) {
+            uint32_t r[LOOK * COPIES], ahead[LOOK * COPIES];       // row numbers of LOOK stages, and of the LOOK after them
+            look_up(0, r);
+            for (uint32_t stage0 = 0; stage0 < stages + CHAIN_STAGES - 1; stage0 += LOOK) {
+                look_up(stage0 + LOOK, ahead);
+#pragma unroll
+                for (uint32_t l = 0; l < LOOK; ++l) {
+                    const uint32_t stage = stage0 + l;
+                    if (stage >= CHAIN_STAGES - 1 && stage < stages + CHAIN_STAGES - 1) {
+                        asm volatile("cp.async.wait_group %0;" ::"n"(CHAIN_STAGES - 2) : "memory");
+                        __syncthreads();                           // stage - (CHAIN_STAGES - 1) is there, the one before it added up
+                    }
+                    const uint32_t to = ring_s + stage % CHAIN_STAGES * CHAIN_STAGE_BYTES + t * 16;
+#pragma unroll
+                    for (uint32_t k = 0; k < COPIES; ++k)
+                        if (r[l * COPIES + k] != 0xFFFFFFFFu)
+                            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to + k * 2048), "l"(src + (uint64_t)r[l * COPIES + k] * L4) : "memory");
+                    asm volatile("cp.async.commit_group;" ::: "memory");
+                }
+#pragma unroll
+                for (uint32_t k = 0; k < LOOK * COPIES; ++k) r[k] = ahead[k];
+            }
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+        }
+        if (adds)
+        for (uint32_t stage = 0; stage < stages; ++stage) {
+            __syncthreads();
+            const V* x = reinterpret_cast<const V*>(ring + stage % CHAIN_STAGES * CHAIN_STAGE_BYTES) + lane;
+            const uint32_t left = min(rows - stage * ROWS, ROWS);
+            uint32_t r = 0;
+            if (left == ROWS) {
+                constexpr uint32_t B = 16;                         // the next rows leave shared memory while these are added
+                V y[2][B];
+#pragma unroll
+                for (uint32_t k = 0; k < B; ++k) y[0][k] = x[k * 32];
+#pragma unroll
+                for (uint32_t b = 0; b < ROWS / B; ++b) {
+                    if (b + 1 < ROWS / B) {
+#pragma unroll
+                        for (uint32_t k = 0; k < B; ++k) y[(b + 1) & 1][k] = x[((b + 1) * B + k) * 32];
+                    }
+#pragma unroll
+                    for (uint32_t k = 0; k < B; ++k) acc += y[b & 1][k];
+                }
+                r = ROWS;
+            }
+            for (; r + 8 <= left; r += 8) {
+                V y[8];
+#pragma unroll
+                for (uint32_t k = 0; k < 8; ++k) y[k] = x[(r + k) * 32];
+#pragma unroll
+                for (uint32_t k = 0; k < 8; ++k) acc += y[k];
+            }
+            for (; r < left; ++r) acc += x[r * 32];
+        }
+        __syncthreads();
+        if (mine) *out = acc;
     }
-    uint64_t end = j + 1;
-    while (end < n && dest[end] == d) ++end;
-    for (uint32_t c = lane; c < L4; c += 32) {
-        float4 a = dv ? tv[c] : make_float4(0.f, 0.f, 0.f, 0.f);
-        float4 b = da ? ta[c] : make_float4(0.f, 0.f, 0.f, 0.f);
-        uint64_t p = j;
-        for (; p + 4 <= end; p += 4) {               // loads issued together, adds kept in order
-            uint64_t o0 = (uint64_t)idx[p] * L4 + c, o1 = (uint64_t)idx[p + 1] * L4 + c;
-            uint64_t o2 = (uint64_t)idx[p + 2] * L4 + c, o3 = (uint64_t)idx[p + 3] * L4 + c;
-            if (dv) {
-                float4 x0 = dv[o0], x1 = dv[o1], x2 = dv[o2], x3 = dv[o3];
-                a = add_chunk<F64>(add_chunk<F64>(add_chunk<F64>(add_chunk<F64>(a, x0), x1), x2), x3);
+}
+
+// Few rows: every block works out all rows' destinations (into shared memory), a warp per row looks whether an earlier row
+// has the same destination and, if none has, finds the later ones by scanning, 32 rows at a step, and adds them in order.
+// One launch in place of seven; the scans grow with n^2.  Measured: 100 rows 15 us (72 us before), 3,000 rows of 64 floats
+// 28 us, while the sort and what follows it take 37 us for 4,500 rows, and a frequent key's chain is slower here (2,500
+// rows, a third of them of one key: 73 us): the line lies at 3,072.
+constexpr uint32_t SMALL_PUSH_ROWS = 3072;
+constexpr unsigned SMALL_THREADS = 256, SMALL_LIST = 512;
+static_assert(SMALL_PUSH_ROWS <= 65536, "row numbers are kept in 16 bits");
+
+template <bool HOT, bool F64>
+__global__ void __launch_bounds__(SMALL_THREADS)
+push_small_kernel(PushDest<uint32_t, HOT> source, uint32_t n, const float4* __restrict__ dv, const float4* __restrict__ da)
+{
+    grid_dependency_wait();
+    constexpr unsigned FULL = 0xFFFFFFFFu;
+    constexpr int U = 16;                                          // rows in flight
+    __shared__ uint32_t dest[SMALL_PUSH_ROWS];
+    __shared__ uint16_t list[SMALL_THREADS / 32][SMALL_LIST];
+    const View& v = source.v;
+    const uint32_t L4 = v.L4, invalid = source.invalid();
+    const uint32_t lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    source.note = blockIdx.x == 0;
+    for (uint32_t b = 0; b < n; b += 4 * SMALL_THREADS) {
+        uint32_t d[4];
+        source(b + threadIdx.x, SMALL_THREADS, n, d);
+#pragma unroll
+        for (int m = 0; m < 4; ++m)
+            if (b + threadIdx.x + m * SMALL_THREADS < n) dest[b + threadIdx.x + m * SMALL_THREADS] = d[m];
+    }
+    __syncthreads();
+    const uint32_t nwarps = gridDim.x * (SMALL_THREADS / 32);
+    for (uint32_t i = (blockIdx.x * SMALL_THREADS + threadIdx.x) >> 5; i < n; i += nwarps) {
+        const uint32_t d = dest[i];
+        if (d == invalid) continue;
+        bool first = true;
+        for (uint32_t b = 0; b < i && first; b += 128) {
+            bool same = false;
+#pragma unroll
+            for (uint32_t k = 0; k < 4; ++k) {
+                const uint32_t j = b + 32 * k + lane;
+                same = same || (j < i && dest[j] == d);
             }
-            if (da) {
-                float4 y0 = da[o0], y1 = da[o1], y2 = da[o2], y3 = da[o3];
-                b = add_chunk<F64>(add_chunk<F64>(add_chunk<F64>(add_chunk<F64>(b, y0), y1), y2), y3);
+            first = !__any_sync(FULL, same);
+        }
+        if (!first) continue;
+        // its rows, up to SMALL_LIST at a time
+        for (uint32_t b = i & ~31u; b < n;) {
+            uint32_t got = 0;
+            for (; b < n && got + 32 <= SMALL_LIST; b += 32) {
+                const uint32_t j = b + lane;
+                const bool member = j >= i && j < n && dest[j] == d;
+                const unsigned m = __ballot_sync(FULL, member);
+                if (member) list[wib][got + __popc(m & ((1u << lane) - 1u))] = (uint16_t)j;
+                got += __popc(m);
             }
+            __syncwarp();
+#pragma unroll
+            for (int which = 0; which < 2; ++which) {
+                const float4* src = which ? da : dv;
+                if (!src) continue;
+                if (got > U)                                       // a chain: all of its rows start towards L2
+                    for (uint32_t e = lane; e < got; e += 32)
+                        for (uint32_t c = 0; c < L4; c += 8) prefetch_l2(src + (uint64_t)list[wib][e] * L4 + c);
+                float4* row = dest_row<uint32_t>(v, d, which);
+                for (uint32_t c = lane; c < L4; c += 32) {
+                    float4 a = row[c];
+                    for (uint32_t e = 0; e < got; e += U) {
+                        float4 x[U];
+#pragma unroll
+                        for (int u = 0; u < U; ++u)
+                            if (e + u < got) x[u] = ld_stream_v4(src + (uint64_t)list[wib][e + u] * L4 + c);
+#pragma unroll
+                        for (int u = 0; u < U; ++u)
+                            if (e + u < got) a = add_chunk<F64>(a, x[u]);
+                    }
+                    row[c] = a;
+                }
+            }
+            __syncwarp();
         }
-        for (; p < end; ++p) {
-            uint64_t o = (uint64_t)idx[p] * L4 + c;
-            if (dv) a = add_chunk<F64>(a, dv[o]);
-            if (da) b = add_chunk<F64>(b, da[o]);
-        }
-        if (dv) tv[c] = a;
-        if (da) ta[c] = b;
     }
 }
 
@@ -945,10 +1227,15 @@ static int bits_for(unsigned long long maxval)
     return b;
 }
 
+// can destinations be numbered with 32 bits?
+static bool narrow_dest(const nups_store* s) { return s->num_keys + (uint64_t)s->R * s->H < 0xFFFFFFFFull; }
+static unsigned long long invalid_dest(const nups_store* s) { return s->num_keys + (uint64_t)s->R * s->H; }
+
 size_t nups_push_scratch_bytes(const nups_store* s, uint64_t n)
 {
     if (!s->cfg.deterministic) return 0;
-    return 2 * align256(n * 8) + 2 * align256(n * 4) + nups_sort_scratch_bytes(n);
+    const size_t key = narrow_dest(s) ? 4 : 8;
+    return 2 * align256(n * key) + 2 * align256(n * 4) + align256((sort_plan(n, bits_for(invalid_dest(s))).hist_words() + 1) * 4);
 }
 
 nups_status nups_push_internal(nups_store* s, const uint32_t* d_keys, uint64_t n, uint32_t rows_per_item,
@@ -960,6 +1247,53 @@ nups_status nups_push_internal(nups_store* s, const uint32_t* d_keys, uint64_t n
         if (rc != NUPS_OK) return rc;
     }
     return nups_push_with_scratch(s, d_keys, n, rows_per_item, d_dval, d_dacc, sc, st);
+}
+
+template <class K, bool HOT>
+static nups_status push_ordered(nups_store* s, const View& v, const uint32_t* d_keys, uint64_t n, uint64_t n_items,
+                                uint32_t rows_per_item, const float* d_dval, const float* d_dacc, char* sc, cudaStream_t st)
+{
+    const float4 *dv = (const float4*)d_dval, *da = (const float4*)d_dacc;
+    const bool f64 = s->vb == 8;
+    PushDest<K, HOT> source = {v, d_keys, n_items, rows_per_item, true};
+    if constexpr (sizeof(K) == 4) {
+        if (n <= SMALL_PUSH_ROWS) {
+            const unsigned grid = grid_for(n, SMALL_THREADS / 32, (unsigned)s->sm_count * 4);
+            if (f64) nups_launch_dependent(push_small_kernel<HOT, true>, grid, SMALL_THREADS, 0, st, source, (uint32_t)n, dv, da);
+            else nups_launch_dependent(push_small_kernel<HOT, false>, grid, SMALL_THREADS, 0, st, source, (uint32_t)n, dv, da);
+            LAUNCH_CHECK(s);
+            return NUPS_OK;
+        }
+    }
+    const K invalid = (K)invalid_dest(s);
+    const SortPlan plan = sort_plan(n, bits_for(invalid));
+    K* k0 = (K*)sc; sc += align256(n * sizeof(K));
+    K* k1 = (K*)sc; sc += align256(n * sizeof(K));
+    uint32_t* v0 = (uint32_t*)sc; sc += align256(n * 4);
+    uint32_t* v1 = (uint32_t*)sc; sc += align256(n * 4);
+    uint32_t* hist = (uint32_t*)sc;
+    nups_launch_dependent(sort_begin_kernel<K, PushDest<K, HOT>>, plan.tiles, SORT_THREADS, 0, st, source, k0, hist, plan);
+    LAUNCH_CHECK(s);
+    K* dest;
+    uint32_t* idx;
+    nups_status rc = sort_passes<K>(s, k0, v0, k1, v1, hist, plan, st, &dest, &idx);
+    if (rc != NUPS_OK) return rc;
+    uint32_t* longs = (uint32_t*)(dest == k0 ? k1 : k0);           // the other key buffer is free now
+    uint32_t* long_count = hist + plan.hist_words();
+#define NUPS_APPLY(F64_, W_)                                                                                              \
+    nups_launch_dependent(push_apply_kernel<K, F64_, W_>, grid_for(n, APPLY_THREADS / 32 * APPLY_WINDOW<W_>), APPLY_THREADS, 0, st, v, (const K*)dest, (const uint32_t*)idx, n, \
+                          invalid, dv, da, longs, long_count)
+    if (f64) { if (v.L4 <= 8) NUPS_APPLY(true, 8); else if (v.L4 <= 16) NUPS_APPLY(true, 16); else NUPS_APPLY(true, 32); }
+    else { if (v.L4 <= 8) NUPS_APPLY(false, 8); else if (v.L4 <= 16) NUPS_APPLY(false, 16); else NUPS_APPLY(false, 32); }
+#undef NUPS_APPLY
+    LAUNCH_CHECK(s);
+    const unsigned chains = (unsigned)s->sm_count * 4;             // 48 KB of shared memory each: four per multiprocessor
+    if (n > APPLY_ROWS) {
+        if (f64) nups_launch_dependent(push_chain_kernel<K, true>, chains, CHAIN_THREADS, CHAIN_SMEM, st, v, (const K*)dest, (const uint32_t*)idx, n, dv, da, (const uint32_t*)longs, (const uint32_t*)long_count);
+        else nups_launch_dependent(push_chain_kernel<K, false>, chains, CHAIN_THREADS, CHAIN_SMEM, st, v, (const K*)dest, (const uint32_t*)idx, n, dv, da, (const uint32_t*)longs, (const uint32_t*)long_count);
+        LAUNCH_CHECK(s);
+    }
+    return NUPS_OK;
 }
 
 nups_status nups_push_with_scratch(nups_store* s, const uint32_t* d_keys, uint64_t n, uint32_t rows_per_item,
@@ -1020,28 +1354,10 @@ nups_status nups_push_with_scratch(nups_store* s, const uint32_t* d_keys, uint64
         LAUNCH_CHECK(s);
         return NUPS_OK;
     }
-    unsigned long long invalid_dest = s->H ? (1ull << 32) + (unsigned long long)s->R * s->H : s->num_keys;
-    int bits = bits_for(invalid_dest);
-    nups_status rc;
-    unsigned long long* k0 = (unsigned long long*)sc; sc += align256(n * 8);
-    unsigned long long* k1 = (unsigned long long*)sc; sc += align256(n * 8);
-    uint32_t* v0 = (uint32_t*)sc; sc += align256(n * 4);
-    uint32_t* v1 = (uint32_t*)sc; sc += align256(n * 4);
-    if (s->H)
-        push_dest_kernel<true><<<grid_for(n, 256), 256, 0, st>>>(v, d_keys, n, n_items, rows_per_item, invalid_dest, k0, v0);
-    else
-        push_dest_kernel<false><<<grid_for(n, 256), 256, 0, st>>>(v, d_keys, n, n_items, rows_per_item, invalid_dest, k0, v0);
-    LAUNCH_CHECK(s);
-    rc = nups_sort_pairs(s, k0, v0, k1, v1, n, bits, sc, st);
-    if (rc != NUPS_OK) return rc;
-    if (s->vb == 8)
-        push_ordered_kernel<true><<<grid_for(n * 32, 256), 256, 0, st>>>(v, k1, v1, n, invalid_dest, (const float4*)d_dval,
-                                                                         (const float4*)d_dacc);
-    else
-        push_ordered_kernel<false><<<grid_for(n * 32, 256), 256, 0, st>>>(v, k1, v1, n, invalid_dest, (const float4*)d_dval,
-                                                                          (const float4*)d_dacc);
-    LAUNCH_CHECK(s);
-    return NUPS_OK;
+    if (narrow_dest(s)) return s->H ? push_ordered<uint32_t, true>(s, v, d_keys, n, n_items, rows_per_item, d_dval, d_dacc, sc, st)
+                                    : push_ordered<uint32_t, false>(s, v, d_keys, n, n_items, rows_per_item, d_dval, d_dacc, sc, st);
+    return s->H ? push_ordered<unsigned long long, true>(s, v, d_keys, n, n_items, rows_per_item, d_dval, d_dacc, sc, st)
+                : push_ordered<unsigned long long, false>(s, v, d_keys, n, n_items, rows_per_item, d_dval, d_dacc, sc, st);
 }
 
 extern "C" nups_status nups_push2(nups_store* s, const uint32_t* d_keys, uint64_t n, const void* d_dval_,
