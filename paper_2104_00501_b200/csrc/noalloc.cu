@@ -6,7 +6,7 @@
 
 // Scratch of nups_push_noalloc.  Every GPU that loads the library holds these bytes until
 // the process exits.  Sized for NUPS_NOALLOC_MAX_ROWS rows: two key buffers, two index
-// buffers, the radix histogram and its scan levels.
+// buffers and the digit counts of the sort.
 #define NUPS_NOALLOC_SCRATCH_BYTES (2u << 20)
 static __device__ __align__(256) unsigned char g_noalloc_scratch[NUPS_NOALLOC_SCRATCH_BYTES];
 

@@ -207,13 +207,9 @@ uint64_t nups_background_merges(nups_store* s);
 
 // primitives.cu
 size_t nups_scan_scratch_bytes(uint64_t n);
-size_t nups_sort_scratch_bytes(uint64_t n);
 // Exclusive prefix sum of n uint64 values (in place allowed); *d_total (device, nullable) receives the sum.
 nups_status nups_scan_u64(nups_store* s, const unsigned long long* d_in, unsigned long long* d_out, uint64_t n,
                           unsigned long long* d_total, char* scratch, cudaStream_t st);
-// Stable LSD radix sort of (key, value) pairs on the low `bits` bits; result ends up in (k_out, v_out).
-nups_status nups_sort_pairs(nups_store* s, unsigned long long* k_in, uint32_t* v_in, unsigned long long* k_out,
-                            uint32_t* v_out, uint64_t n, int bits, char* scratch, cudaStream_t st);
 
 // store.cu internals used by steps.cu / sampling.cu
 // (value buffers are passed as float* whatever the value type: storage, counted in 4-byte units)

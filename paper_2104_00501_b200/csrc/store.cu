@@ -1472,84 +1472,279 @@ extern "C" nups_status nups_sync(nups_store* s, void* stream)
 // ---------------------------------------------------------------------------------------------
 // access counting and hot-set selection
 // ---------------------------------------------------------------------------------------------
-__global__ void count_kernel(View v, const uint32_t* __restrict__ keys, uint64_t n)
+// A block adds up the keys it meets again in shared memory: a table of COUNT_SLOTS keys and counts, a slot belonging to the
+// first key that asks for it.  Frequent keys show up early, so they take slots, and thousands of additions no longer queue
+// at one address; all other keys are counted by one reduction each.  (Looking for equal keys within a warp by a match
+// instruction took longer than the reductions that it saved.)  Two blocks per multiprocessor.  Measured, 4M keys over 11M:
+// 79 -> 47 us at Zipf 0.8, 155 -> 34 us at Zipf 1.0 (launch and events included).
+constexpr unsigned COUNT_THREADS = 1024, COUNT_SLOT_BITS = 12, COUNT_SLOTS = 1u << COUNT_SLOT_BITS, COUNT_ITEMS = 4;
+
+__global__ void __launch_bounds__(COUNT_THREADS)
+count_kernel(View v, const uint32_t* __restrict__ keys, uint64_t n)
 {
-    uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const unsigned lane = threadIdx.x & 31;
-    bool in = i < n;
-    uint32_t key = in ? keys[i] : 0u;
-    bool valid = in && key < v.num_keys;
-    if (in && !valid) flag_bad_key(v);
-    unsigned long long tag = valid ? (unsigned long long)key : (~0ull - lane);
-    unsigned grp = __match_any_sync(0xFFFFFFFFu, tag);
-    if (valid && lane == (unsigned)(__ffs(grp) - 1)) atomicAdd(v.cnt + key, (unsigned long long)__popc(grp));
+    __shared__ uint32_t tag[COUNT_SLOTS], count[COUNT_SLOTS];
+    for (unsigned e = threadIdx.x; e < COUNT_SLOTS; e += COUNT_THREADS) { tag[e] = NUPS_INVALID_KEY; count[e] = 0u; }
+    __syncthreads();
+    const uint64_t step = (uint64_t)gridDim.x * COUNT_THREADS;
+    for (uint64_t i = (uint64_t)blockIdx.x * COUNT_THREADS + threadIdx.x; i < n; i += COUNT_ITEMS * step) {
+        uint32_t k[COUNT_ITEMS];
+#pragma unroll
+        for (int m = 0; m < (int)COUNT_ITEMS; ++m) k[m] = i + m * step < n ? __ldcs(keys + i + m * step) : NUPS_INVALID_KEY;
+#pragma unroll
+        for (int m = 0; m < (int)COUNT_ITEMS; ++m) {
+            if (k[m] >= v.num_keys) {                        // the largest 32-bit number is never a key
+                if (i + m * step < n) flag_bad_key(v);
+                continue;
+            }
+            const unsigned at = (k[m] * 0x9E3779B1u) >> (32 - COUNT_SLOT_BITS);
+            uint32_t owner = tag[at];
+            if (owner == NUPS_INVALID_KEY) {
+                owner = atomicCAS(&tag[at], NUPS_INVALID_KEY, k[m]);
+                if (owner == NUPS_INVALID_KEY) owner = k[m];
+            }
+            if (owner == k[m]) atomicAdd(&count[at], 1u);
+            else atomicAdd(v.cnt + k[m], 1ull);
+        }
+    }
+    __syncthreads();
+    for (unsigned e = threadIdx.x; e < COUNT_SLOTS; e += COUNT_THREADS)
+        if (count[e]) atomicAdd(v.cnt + tag[e], (unsigned long long)count[e]);
 }
 
 extern "C" nups_status nups_count_accesses(nups_store* s, const uint32_t* d_keys, uint64_t n, void* stream)
 {
     if (!s || (n && !d_keys)) return NUPS_EINVAL;
     if (n == 0) return NUPS_OK;
-    count_kernel<<<grid_for(n, 256), 256, 0, (cudaStream_t)stream>>>(nups_view(s), d_keys, n);
+    count_kernel<<<grid_for(n, COUNT_THREADS, (unsigned)s->sm_count * 2), COUNT_THREADS, 0, (cudaStream_t)stream>>>(nups_view(s), d_keys, n);
     LAUNCH_CHECK(s);
     return NUPS_OK;
+}
+
+// The counts are handed out by a copy of our own: they are next to the multiprocessors in L2 when they have just been
+// counted or chosen from, and reading 64 bytes per thread at once takes them out faster than the copy call (88 MB: 42 us, 50 us).
+__global__ void __launch_bounds__(256)
+copy_counts_kernel(const ulonglong2* __restrict__ from, ulonglong2* __restrict__ to, uint64_t n2)
+{
+    const uint64_t first = (uint64_t)blockIdx.x * 1024 + threadIdx.x;
+    ulonglong2 x[4];
+#pragma unroll
+    for (int m = 0; m < 4; ++m)
+        if (first + m * 256 < n2) x[m] = __ldcg(from + first + m * 256);
+#pragma unroll
+    for (int m = 0; m < 4; ++m)
+        if (first + m * 256 < n2) __stcs(to + first + m * 256, x[m]);
 }
 
 extern "C" nups_status nups_get_counts(nups_store* s, uint64_t* d_out, void* stream)
 {
     if (!s || !d_out) return NUPS_EINVAL;
-    CK(cudaMemcpyAsync(d_out, s->cnt, s->num_keys * 8, cudaMemcpyDeviceToDevice, (cudaStream_t)stream));
+    cudaStream_t st = (cudaStream_t)stream;
+    if ((uintptr_t)d_out & 15) {                             // not aligned for wide stores
+        CK(cudaMemcpyAsync(d_out, s->cnt, s->num_keys * 8, cudaMemcpyDeviceToDevice, st));
+        return NUPS_OK;
+    }
+    const uint64_t n2 = s->num_keys / 2;
+    if (n2) {
+        copy_counts_kernel<<<grid_for(n2, 1024), 256, 0, st>>>((const ulonglong2*)s->cnt, (ulonglong2*)d_out, n2);
+        LAUNCH_CHECK(s);
+    }
+    if (s->num_keys & 1) CK(cudaMemcpyAsync(d_out + 2 * n2, s->cnt + 2 * n2, 8, cudaMemcpyDeviceToDevice, st));
     return NUPS_OK;
 }
 
-__global__ void count_sum_max_kernel(const unsigned long long* __restrict__ cnt, uint64_t n, DevStat* st)
+// Choosing the hot keys.  Only the keys that are chosen are ever sorted:
+//   1. one pass over the counts: their sum, their maximum, and how many lie in each of 976 bins (exact below 32, sixteen
+//      bins per power of two above).  The host reads these and knows the lowest count that is chosen, or the bin it is in;
+//      a bin that holds many more keys than are wanted is cut finer by further passes;
+//   2. per stretch of keys, how many lie above that count and on it; their prefix sums;
+//   3. the chosen keys in key order (of those on the lowest count, the first ones), and a stable sort by count.
+// Measured, the 10,000 most frequent of 11M keys: 117 us of kernels (bins 41, stretches 32, prefix sums 6, chosen keys 7, sort 25),
+// where a sort of all keys by count and key took 1,400.
+constexpr unsigned SELECT_THREADS = 256, SELECT_BINS = 1024, SELECT_MAX_RANGES = 2048;
+constexpr uint64_t SELECT_CHUNK = 8 * SELECT_THREADS;
+
+struct CountStat {
+    unsigned long long sum, max;
+    unsigned long long bin[SELECT_BINS];
+};
+
+__device__ __forceinline__ unsigned count_bin(unsigned long long c)
 {
-    uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+    if (c < 32) return (unsigned)c;
+    const unsigned e = 63u - (unsigned)__clzll((long long)c);
+    return 32u + (e - 5u) * 16u + (unsigned)((c >> (e - 4u)) & 15u);
+}
+// smallest count of a bin, and how many counts it spans (as a power of two)
+static unsigned long long bin_first(unsigned b) { return b < 32 ? b : (unsigned long long)(16 + (b - 32) % 16) << ((b - 32) / 16 + 1); }
+static unsigned bin_shift(unsigned b) { return b < 32 ? 0 : (b - 32) / 16 + 1; }
+
+// FIRST: sum, maximum and the bins of count_bin.  Otherwise: the counts c with first <= c, (c - first) >> shift < SELECT_BINS.
+template <bool FIRST>
+__global__ void __launch_bounds__(SELECT_THREADS)
+count_stat_kernel(const unsigned long long* __restrict__ cnt, uint64_t n, unsigned long long first, unsigned shift,
+                  CountStat* __restrict__ out)
+{
+    constexpr unsigned COPIES = 4;                           // lanes of a warp that meet in a bin are spread over these
+    __shared__ __align__(16) unsigned h[SELECT_BINS * COPIES];
+    for (unsigned e = threadIdx.x; e < SELECT_BINS * COPIES; e += SELECT_THREADS) h[e] = 0u;
+    __syncthreads();
+    unsigned* mine = h + threadIdx.x % COPIES;
     unsigned long long sum = 0, mx = 0;
-    for (; i < n; i += stride) {
-        unsigned long long c = cnt[i];
-        sum += c;
-        mx = c > mx ? c : mx;
+    unsigned zeros = 0, ones = 0;                            // most keys: counted in registers
+    auto take = [&](unsigned long long c) {
+        if (FIRST) {
+            sum += c;
+            mx = c > mx ? c : mx;
+            if (c == 0) ++zeros;
+            else if (c == 1) ++ones;
+            else atomicAdd(mine + COPIES * count_bin(c), 1u);
+        } else if (c >= first && (c - first) >> shift < SELECT_BINS) {
+            atomicAdd(mine + COPIES * (unsigned)((c - first) >> shift), 1u);
+        }
+    };
+    const uint64_t pairs = n / 2, step = (uint64_t)gridDim.x * SELECT_THREADS;
+    const ulonglong2* two = reinterpret_cast<const ulonglong2*>(cnt);
+    for (uint64_t i = (uint64_t)blockIdx.x * SELECT_THREADS + threadIdx.x; i < pairs; i += 4 * step) {
+        ulonglong2 c[4];
+#pragma unroll
+        for (int m = 0; m < 4; ++m)
+            if (i + m * step < pairs) c[m] = two[i + m * step];
+#pragma unroll
+        for (int m = 0; m < 4; ++m)
+            if (i + m * step < pairs) { take(c[m].x); take(c[m].y); }
     }
-    for (int o = 16; o > 0; o >>= 1) {
-        sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
-        unsigned long long m2 = __shfl_xor_sync(0xFFFFFFFFu, mx, o);
-        mx = m2 > mx ? m2 : mx;
+    if ((n & 1) && blockIdx.x == 0 && threadIdx.x == 0) take(cnt[n - 1]);
+    if (FIRST) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
+            const unsigned long long m2 = __shfl_xor_sync(0xFFFFFFFFu, mx, o);
+            mx = m2 > mx ? m2 : mx;
+            zeros += __shfl_xor_sync(0xFFFFFFFFu, zeros, o);
+            ones += __shfl_xor_sync(0xFFFFFFFFu, ones, o);
+        }
+        if ((threadIdx.x & 31) == 0) {
+            atomicAdd(&out->sum, sum);
+            atomicMax(&out->max, mx);
+            if (zeros) atomicAdd(h, zeros);
+            if (ones) atomicAdd(h + COPIES, ones);
+        }
     }
-    if ((threadIdx.x & 31) == 0) {
-        atomicAdd(&st->tmp[0], sum);
-        atomicMax(&st->tmp[1], mx);
+    __syncthreads();
+    for (unsigned e = threadIdx.x; e < SELECT_BINS; e += SELECT_THREADS) {
+        const uint4 x = reinterpret_cast<const uint4*>(h)[e];
+        const unsigned long long all = (unsigned long long)x.x + x.y + x.z + x.w;
+        if (all) atomicAdd(&out->bin[e], all);
     }
 }
 
-// flag[k] = 1 when key k is selected by the threshold rule cnt*num_keys > factor*total (exact)
-__global__ void threshold_flag_kernel(const unsigned long long* __restrict__ cnt, uint64_t n, unsigned long long factor,
-                                      unsigned long long total, unsigned long long* __restrict__ flag)
+// Keys of a stretch with a count above `cut` (upper half of the word) and on it (lower half).  Two words of bits per 64 keys
+// say which ones have either: the even and the odd ones.
+__global__ void __launch_bounds__(SELECT_THREADS)
+select_count_kernel(const unsigned long long* __restrict__ cnt, uint64_t n, uint64_t range, unsigned long long cut,
+                    unsigned long long* __restrict__ found, uint2* __restrict__ bits)
 {
-    uint64_t k = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n) return;
-    unsigned long long c = cnt[k];
-    unsigned long long lhi = __umul64hi(c, n), llo = c * n;
-    unsigned long long rhi = __umul64hi(factor, total), rlo = factor * total;
-    flag[k] = (lhi > rhi || (lhi == rhi && llo > rlo)) ? 1ull : 0ull;
+    constexpr unsigned FULL = 0xFFFFFFFFu;
+    __shared__ unsigned long long total;
+    if (threadIdx.x == 0) total = 0;
+    __syncthreads();
+    const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint64_t first = blockIdx.x * range, last = min(first + range, n);
+    unsigned above = 0, either = 0;
+    for (uint64_t b = first; b < last; b += SELECT_CHUNK) {              // a stretch is a whole number of chunks
+        ulonglong2 c[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {                                    // a warp looks at 256 consecutive counts
+            const uint64_t i = b + warp * 256 + k * 64 + lane * 2;
+            c[k] = make_ulonglong2(0, 0);
+            if (i + 1 < last) c[k] = *reinterpret_cast<const ulonglong2*>(cnt + i);
+            else if (i < last) c[k].x = cnt[i];
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const uint64_t i = b + warp * 256 + k * 64 + lane * 2;
+            const bool x = i < last && c[k].x >= cut, y = i + 1 < last && c[k].y >= cut;
+            const uint2 w = make_uint2(__ballot_sync(FULL, x), __ballot_sync(FULL, y));
+            if (lane == 0 && i < last) bits[i >> 6] = w;
+            above += (x && c[k].x > cut) + (y && c[k].y > cut);
+            either += x + y;
+        }
+    }
+    unsigned long long both = (unsigned long long)above << 32 | (either - above);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) both += __shfl_xor_sync(FULL, both, o);
+    if (lane == 0) atomicAdd(&total, both);
+    __syncthreads();
+    if (threadIdx.x == 0) found[blockIdx.x] = total;
 }
 
-// composite sort key: (max_cnt - cnt) in the high part, key in the low `key_bits` bits, so that an
-// ascending sort gives count descending, key ascending
-__global__ void composite_kernel(const unsigned long long* __restrict__ cnt, uint64_t n, unsigned long long max_cnt,
-                                 int key_bits, const unsigned long long* __restrict__ flag /* nullable */,
-                                 const unsigned long long* __restrict__ pos /* exclusive scan of flag */,
-                                 unsigned long long* __restrict__ comp, uint32_t* __restrict__ payload)
+// The chosen keys and their counts in key order: all keys above `cut` and the first `ties` of those on it.  `before` = for
+// every stretch, the keys above (upper half) and on the cut in the stretches before it.  A thread takes 64 keys and reads
+// the counts of those whose bit is set only.
+__global__ void __launch_bounds__(SELECT_THREADS)
+select_write_kernel(const unsigned long long* __restrict__ cnt, uint64_t n, uint64_t range, unsigned long long cut,
+                    unsigned long long ties, const unsigned long long* __restrict__ before, const uint2* __restrict__ bits,
+                    uint32_t* __restrict__ keys, unsigned long long* __restrict__ counts)
 {
-    uint64_t k = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n) return;
-    uint64_t o = k;
-    if (flag) {
-        if (!flag[k]) return;
-        o = pos[k];
+    __shared__ unsigned long long warp_sum[SELECT_THREADS / 32];
+    const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint64_t first = blockIdx.x * range, last = min(first + range, n);
+    unsigned long long so_far = before[blockIdx.x];
+    for (uint64_t b = first; b < last; b += 64 * SELECT_THREADS) {
+        const uint64_t i = b + 64 * threadIdx.x;
+        const uint2 w = i < last ? bits[i >> 6] : make_uint2(0u, 0u);
+        auto each = [&](auto use) {                          // the thread's keys in order
+            for (unsigned left = w.x | w.y; left; left &= left - 1) {
+                const unsigned at = __ffs(left) - 1;
+                if (w.x >> at & 1u) use(i + 2 * at, cnt[i + 2 * at]);
+                if (w.y >> at & 1u) use(i + 2 * at + 1, cnt[i + 2 * at + 1]);
+            }
+        };
+        unsigned long long mine = 0;
+        each([&](uint64_t, unsigned long long c) { mine += c > cut ? 1ull << 32 : 1ull; });
+        unsigned long long inc = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+            if (lane >= (unsigned)o) inc += y;
+        }
+        __syncthreads();                                     // the round before's readers are done
+        if (lane == 31) warp_sum[warp] = inc;
+        __syncthreads();
+        unsigned long long here = so_far + inc - mine;
+        for (unsigned k = 0; k < SELECT_THREADS / 32; ++k) {
+            if (k < warp) here += warp_sum[k];
+            so_far += warp_sum[k];
+        }
+        each([&](uint64_t key, unsigned long long c) {
+            const unsigned long long above = here >> 32, on = here & 0xFFFFFFFFull;
+            if (c > cut || on < ties) {
+                const unsigned long long at = above + (on < ties ? on : ties);
+                keys[at] = (uint32_t)key;
+                counts[at] = c;
+            }
+            here += c > cut ? 1ull << 32 : 1ull;
+        });
     }
-    comp[o] = ((max_cnt - cnt[k]) << key_bits) | k;
-    payload[o] = (uint32_t)k;
+}
+
+// sort keys of the chosen: how far a count lies below the largest one
+struct BelowMax {
+    const unsigned long long* counts;
+    unsigned long long max_cnt;
+    template <int N>
+    __device__ __forceinline__ void operator()(uint64_t i, uint64_t step, uint64_t n, unsigned long long (&d)[N]) const
+    {
+#pragma unroll
+        for (int m = 0; m < N; ++m) d[m] = i + m * step < n ? max_cnt - counts[i + m * step] : 0ull;
+    }
+};
+
+__global__ void select_out_kernel(const uint32_t* __restrict__ keys, const uint32_t* __restrict__ order, uint64_t n, uint32_t* __restrict__ out)
+{
+    grid_dependency_wait();
+    const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) out[i] = keys[order[i]];
 }
 
 extern "C" nups_status nups_select_hot(nups_store* s, int by_topk, uint64_t param, uint32_t* d_keys_out,
@@ -1557,50 +1752,100 @@ extern "C" nups_status nups_select_hot(nups_store* s, int by_topk, uint64_t para
 {
     if (!s || !d_keys_out || !h_n_out) return NUPS_EINVAL;
     cudaStream_t st = (cudaStream_t)stream;
-    uint64_t n = s->num_keys;
+    const uint64_t n = s->num_keys;
     *h_n_out = 0;
-    CK(cudaMemsetAsync(&s->st->tmp[0], 0, 16, st));
-    count_sum_max_kernel<<<grid_for(n, 256, (unsigned)s->sm_count * 8), 256, 0, st>>>(s->cnt, n, s->st);
-    LAUNCH_CHECK(s);
-    unsigned long long sm[2];
-    CK(cudaMemcpyAsync(sm, &s->st->tmp[0], 16, cudaMemcpyDeviceToHost, st));
-    CK(cudaStreamSynchronize(st));
-    unsigned long long total = sm[0], max_cnt = sm[1];
-    int key_bits = bits_for(n - 1), cnt_bits = bits_for(max_cnt);
-    if (key_bits + cnt_bits > 64) return NUPS_ESTATE;
-    size_t need = 4 * align256(n * 8) + 2 * align256(n * 4) + nups_sort_scratch_bytes(n) + nups_scan_scratch_bytes(n) + 256;
+    const uint64_t range = ((n + SELECT_MAX_RANGES - 1) / SELECT_MAX_RANGES + SELECT_CHUNK - 1) / SELECT_CHUNK * SELECT_CHUNK;
+    const unsigned ranges = (unsigned)((n + range - 1) / range);
+    const size_t bits_at = align256(sizeof(CountStat)) + align256(ranges * 8 + 8) + nups_scan_scratch_bytes(ranges);
+    const size_t fixed = bits_at + align256((n + 63) / 64 * 8);
     char* sc;
-    nups_status rc = nups_scratch(s, need, &sc);
+    nups_status rc = nups_scratch(s, fixed, &sc);
     if (rc != NUPS_OK) return rc;
-    unsigned long long* flag = (unsigned long long*)sc; sc += align256(n * 8);
-    unsigned long long* pos = (unsigned long long*)sc; sc += align256(n * 8);
-    unsigned long long* c0 = (unsigned long long*)sc; sc += align256(n * 8);
-    unsigned long long* c1 = (unsigned long long*)sc; sc += align256(n * 8);
-    uint32_t* p0 = (uint32_t*)sc; sc += align256(n * 4);
-    uint32_t* p1 = (uint32_t*)sc; sc += align256(n * 4);
-    unsigned long long* d_m = (unsigned long long*)sc; sc += 256;
-    uint64_t m = n;
-    if (!by_topk) {
-        threshold_flag_kernel<<<grid_for(n, 256), 256, 0, st>>>(s->cnt, n, param, total, flag);
-        LAUNCH_CHECK(s);
-        rc = nups_scan_u64(s, flag, pos, n, d_m, sc, st);
-        if (rc != NUPS_OK) return rc;
-        unsigned long long hm = 0;
-        CK(cudaMemcpyAsync(&hm, d_m, 8, cudaMemcpyDeviceToHost, st));
-        CK(cudaStreamSynchronize(st));
-        m = hm;
-        if (m == 0) return NUPS_OK;
-        composite_kernel<<<grid_for(n, 256), 256, 0, st>>>(s->cnt, n, max_cnt, key_bits, flag, pos, c0, p0);
-    } else {
-        if (param == 0) return NUPS_OK;
-        composite_kernel<<<grid_for(n, 256), 256, 0, st>>>(s->cnt, n, max_cnt, key_bits, nullptr, nullptr, c0, p0);
-    }
+    CountStat* d_stat = (CountStat*)sc;
+    CountStat stat;
+    const unsigned grid = grid_for(n, 8 * SELECT_THREADS, (unsigned)s->sm_count * 8);
+    CK(cudaMemsetAsync(d_stat, 0, sizeof(CountStat), st));
+    count_stat_kernel<true><<<grid, SELECT_THREADS, 0, st>>>(s->cnt, n, 0, 0, d_stat);
     LAUNCH_CHECK(s);
-    char* sort_sc = sc + nups_scan_scratch_bytes(n);
-    rc = nups_sort_pairs(s, c0, p0, c1, p1, m, key_bits + cnt_bits, sort_sc, st);
+    CK(cudaMemcpyAsync(&stat, d_stat, sizeof(stat), cudaMemcpyDeviceToHost, st));
+    CK(cudaStreamSynchronize(st));
+    const unsigned long long total = stat.sum, max_cnt = stat.max;
+    if (bits_for(n - 1) + bits_for(max_cnt) > 64) return NUPS_ESTATE;
+    // keys above `cut` are chosen, and the first `ties` of those on it; m = how many that makes, `take` of them are wanted
+    unsigned long long cut = 0, ties = 0;
+    uint64_t m = 0, take = 0;
+    if (by_topk) {
+        take = param < n ? param : n;
+        if (take == 0) return NUPS_OK;
+        uint64_t above = 0;                                  // keys in higher bins
+        unsigned b = SELECT_BINS - 1;
+        while (above + stat.bin[b] < take) above += stat.bin[b--];
+        unsigned long long first = bin_first(b);
+        unsigned shift = bin_shift(b);
+        // the bin reaches from `first` over 2^shift counts.  Cut it finer while it holds far more keys than are wanted.
+        while (shift && stat.bin[b] > take && stat.bin[b] > 65536) {
+            const unsigned fine = shift > 10 ? shift - 10 : 0;
+            CK(cudaMemsetAsync(d_stat, 0, sizeof(CountStat), st));
+            count_stat_kernel<false><<<grid, SELECT_THREADS, 0, st>>>(s->cnt, n, first, fine, d_stat);
+            LAUNCH_CHECK(s);
+            CK(cudaMemcpyAsync(&stat, d_stat, sizeof(stat), cudaMemcpyDeviceToHost, st));
+            CK(cudaStreamSynchronize(st));
+            b = (unsigned)((1ull << (shift - fine)) - 1);    // the finer bins of the old one only
+            while (above + stat.bin[b] < take) above += stat.bin[b--];
+            first += (unsigned long long)b << fine;
+            shift = fine;
+        }
+        if (shift == 0) { cut = first; ties = take - above; m = take; }
+        else { cut = first - 1; ties = 0; m = above + stat.bin[b]; }         // the whole bin: the sort finds the first `take`
+    } else {
+        // count * n > param * total, exactly: count > floor(param * total / n)
+        const unsigned __int128 q = (unsigned __int128)param * total / n;
+        if (q >= max_cnt) return NUPS_OK;
+        cut = (unsigned long long)q;
+    }
+    unsigned long long* found = (unsigned long long*)(sc + align256(sizeof(CountStat)));
+    auto count_found = [&]() -> nups_status {
+        select_count_kernel<<<ranges, SELECT_THREADS, 0, st>>>(s->cnt, n, range, cut, found, (uint2*)(sc + bits_at));
+        LAUNCH_CHECK(s);
+        return nups_scan_u64(s, found, found, ranges, found + ranges, (char*)found + align256(ranges * 8 + 8), st);
+    };
+    if (!by_topk) {
+        rc = count_found();
+        if (rc != NUPS_OK) return rc;
+        unsigned long long both = 0;
+        CK(cudaMemcpyAsync(&both, found + ranges, 8, cudaMemcpyDeviceToHost, st));
+        CK(cudaStreamSynchronize(st));
+        take = m = both >> 32;
+        if (m == 0) return NUPS_OK;
+    }
+    const SortPlan plan = sort_plan(m, bits_for(max_cnt - cut));
+    const size_t need = fixed + align256(m * 4) * 3 + align256(m * 8) * 3 + align256((plan.hist_words() + 1) * 4);
+    const bool moves = need > s->scratch_bytes;              // a larger buffer: what was found is found again there
+    rc = nups_scratch(s, need, &sc);
     if (rc != NUPS_OK) return rc;
-    uint64_t take = by_topk ? (param < m ? param : m) : m;
-    CK(cudaMemcpyAsync(d_keys_out, p1, take * 4, cudaMemcpyDeviceToDevice, st));
+    found = (unsigned long long*)(sc + align256(sizeof(CountStat)));
+    if (by_topk || moves) rc = count_found();
+    if (rc != NUPS_OK) return rc;
+    const uint2* bits = (const uint2*)(sc + bits_at);
+    sc += fixed;
+    uint32_t* keys = (uint32_t*)sc; sc += align256(m * 4);
+    uint32_t* v0 = (uint32_t*)sc; sc += align256(m * 4);
+    uint32_t* v1 = (uint32_t*)sc; sc += align256(m * 4);
+    unsigned long long* counts = (unsigned long long*)sc; sc += align256(m * 8);
+    unsigned long long* k0 = (unsigned long long*)sc; sc += align256(m * 8);
+    unsigned long long* k1 = (unsigned long long*)sc; sc += align256(m * 8);
+    uint32_t* hist = (uint32_t*)sc;
+    select_write_kernel<<<ranges, SELECT_THREADS, 0, st>>>(s->cnt, n, range, cut, ties, found, bits, keys, counts);
+    LAUNCH_CHECK(s);
+    const BelowMax below = {counts, max_cnt};
+    nups_launch_dependent(sort_begin_kernel<unsigned long long, BelowMax>, plan.tiles, SORT_THREADS, 0, st, below, k0, hist, plan);
+    LAUNCH_CHECK(s);
+    unsigned long long* sorted;
+    uint32_t* order;
+    rc = sort_passes<unsigned long long>(s, k0, v0, k1, v1, hist, plan, st, &sorted, &order);
+    if (rc != NUPS_OK) return rc;
+    nups_launch_dependent(select_out_kernel, grid_for(take, 256), 256, 0, st, keys, order, take, d_keys_out);
+    LAUNCH_CHECK(s);
     CK(cudaStreamSynchronize(st));
     *h_n_out = take;
     return NUPS_OK;

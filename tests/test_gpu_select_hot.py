@@ -1,0 +1,64 @@
+"""Counting and choosing hot keys at the sizes where the parts hand over: the block's own table of keys, bins of counts that
+are cut finer, ties on the lowest chosen count, stretches of keys."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2104_00501_b200 import binding
+from tests.common import dev_keys, host_keys
+
+pytestmark = pytest.mark.gpu
+
+
+def _top(counts, k):
+    return np.lexsort((np.arange(len(counts)), -counts))[:k].astype(np.uint32)
+
+
+def _check(s, counts, tops, factors=()):
+    assert np.array_equal(s.counts().cpu().numpy(), counts)
+    for k in tops:
+        assert np.array_equal(host_keys(s.select_hot(True, k)), _top(counts, k)), k
+    for f in factors:
+        m = int((counts * len(counts) > f * counts.sum()).sum())       # far below 2^63
+        assert np.array_equal(host_keys(s.select_hot(False, f)), _top(counts, m)), f
+
+
+@pytest.mark.parametrize("nk", [1, 2, 2047, 2049, 300_001])
+def test_counts_and_choices_of_every_size(nk):
+    rng = np.random.default_rng(nk)
+    s = binding.Store(nk, 4, sync_interval=0)
+    counts = np.zeros(nk, np.int64)
+    _check(s, counts, [1, nk // 2, nk, nk + 7], [0, 1])               # nothing counted yet: all keys tie
+    for n in (1, 1023, 4097, 700_003):
+        keys = np.where(rng.random(n) < 0.5, rng.zipf(1.3, n) % nk, rng.integers(0, nk, n)).astype(np.uint32)
+        s.count_accesses(dev_keys(keys))
+        counts += np.bincount(keys, minlength=nk)
+        if n in (1, 700_003):
+            _check(s, counts, sorted({1, 2, 10, nk // 3, nk - 1, nk} - {0}), [1, 2, 3, 100])
+    bad = np.array([nk, 0xFFFFFFFF, 0, nk - 1], np.uint32)
+    s.count_accesses(dev_keys(bad))
+    counts[0] += 1
+    counts[nk - 1] += 1
+    _check(s, counts, [1, min(nk, 5)])
+    assert s.status_check() == -4
+    s.close()
+
+
+@pytest.mark.parametrize("calls", [4, 66])
+def test_a_bin_that_holds_too_many_keys_is_cut_finer(calls):
+    # 70,000 keys whose counts share one bin: 10 * calls (+ up to 6) accesses each; 33,000 are cut twice
+    nk, busy = 100_000, 70_000
+    rng = np.random.default_rng(calls)
+    s = binding.Store(nk, 4, sync_interval=0)
+    named = rng.permutation(nk)[:busy].astype(np.uint32)
+    per_call = 10 if calls == 4 else 500
+    keys = dev_keys(np.tile(named, per_call))
+    for _ in range(calls):
+        s.count_accesses(keys)
+    counts = np.zeros(nk, np.int64)
+    counts[named] = per_call * calls
+    more = np.repeat(named, np.arange(busy) % 7)
+    s.count_accesses(dev_keys(more))
+    counts += np.bincount(more, minlength=nk)
+    _check(s, counts, [1, 9_999, 10_001, 40_000, 69_999, 70_001, nk], [1, 2])
+    s.close()
