@@ -1,9 +1,10 @@
-"""Counting and choosing hot keys at the sizes where the parts hand over: the block's own table of keys, bins of counts that
-are cut finer, ties on the lowest chosen count, stretches of keys."""
+"""Counting, choosing and managing hot keys at the sizes where the parts hand over: the block's own table of keys, bins of
+counts that are cut finer, ties on the lowest chosen count, stretches of keys, and lists around the one-block limit."""
 import numpy as np
 import pytest
 import torch
 
+from oracle import REPLICATE, SINGLE, Oracle
 from paper_2104_00501_b200 import binding
 from tests.common import dev_keys, host_keys
 
@@ -61,4 +62,19 @@ def test_a_bin_that_holds_too_many_keys_is_cut_finer(calls):
     s.count_accesses(dev_keys(more))
     counts += np.bincount(more, minlength=nk)
     _check(s, counts, [1, 9_999, 10_001, 40_000, 69_999, 70_001, nk], [1, 2])
+    s.close()
+
+
+@pytest.mark.parametrize("n", [1, 1024, 1025, 4097, 16_384, 16_385, 1_048_577])
+def test_lists_around_the_one_block_limit(n):
+    nk, L = 60_000, 4
+    rng = np.random.default_rng(n)
+    o, s = Oracle(nk, L, workers=3), binding.Store(nk, L, workers=3)
+    for round_ in range(3):
+        up = rng.integers(0, nk, n).astype(np.uint32)                 # repeats included
+        down = np.concatenate([up[rng.random(n) < 0.4], rng.integers(0, nk, 50).astype(np.uint32)])
+        for keys, technique in ((up, (REPLICATE, binding.REPLICATE)), (down, (SINGLE, binding.SINGLE))):
+            o.set_management(keys, technique[0])
+            s.set_management(dev_keys(keys), technique[1])
+            assert np.array_equal(host_keys(s.hot_keys()), o.hot_keys())
     s.close()
