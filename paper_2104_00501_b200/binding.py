@@ -136,7 +136,9 @@ def _ptr(t, dtype=None):
 
 
 def _stream():
-    return torch.cuda.current_stream().cuda_stream
+    # the current device's current stream as a number, without the Stream object that torch.cuda.current_stream() makes
+    # (1.5 us of the 5 us that a small call spends in Python); a Store has initialised CUDA by then
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def as_keys(t) -> torch.Tensor:
