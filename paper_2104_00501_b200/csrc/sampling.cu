@@ -242,7 +242,7 @@ struct HandleView {
     uint4* state;      // LONG-TERM per sub-handle: x = walk position, y = postponed head, z = postponed tail
     uint4* prev;       //   the state before the running call
     uint4* walk;       //   what the running call does: x = fresh entries walked, y = of those local,
-                       //   z = postponed entries emitted
+                       //   z = postponed entries emitted, w = blocks that have looked up their part (0 between calls)
     uint32_t* flags;   // LONG-TERM: "is local" bit of every fresh entry, and the number of local entries before
     uint32_t* prefix;  //   each 32-entry word; sub-handle q owns the words from (b_q / 32) + q on
 };
@@ -499,7 +499,7 @@ __global__ void draw_reuse_kernel(View v, DrawParams p, const unsigned long long
     const unsigned long long s0 = off_cur[q];
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         off_next[q] = s0 + size;
-        if (longterm) h.state[q] = make_uint4(0u, 0u, 0u, 0u);
+        if (longterm) h.state[q] = h.walk[q] = make_uint4(0u, 0u, 0u, 0u);
     }
     if (size == 0) return;
     reuse_pool_visit(p, q, s0, s0 + size, T, [&](bool in, uint32_t k, unsigned long long rel, bool mark) {
@@ -614,9 +614,9 @@ __global__ void emit_kernel(View v, DrawParams p, HandleView h, uint64_t N, uint
 // the walk stops right after the last entry it must emit, and when the fresh entries run out the
 // postponed ones are emitted.  Locality is judged by the ownership at the start of the call.
 // Where an entry goes depends only on how many local entries lie before it, so the walk is a
-// prefix sum, not a loop: (1) one bit per fresh entry, looked up by the whole GPU; (2) per sub-handle,
-// a scan of the bit counts that also finds where the walk stops (and emits entries that earlier calls
-// postponed); (3) every entry is placed on its own, and what is postponed moves to its worker.
+// prefix sum, not a loop: one bit per fresh entry, looked up by the whole GPU; per sub-handle, a scan of the bit
+// counts that also finds where the walk stops, made by the block that is the last to have looked up its part; then
+// every entry is placed on its own, and what is postponed moves to its worker.
 struct LtChunk {
     uint32_t q;
     uint64_t b0, size, take, out_base;
@@ -636,41 +636,49 @@ __device__ __forceinline__ LtChunk lt_chunk(uint32_t q, uint64_t N, uint32_t R, 
     return c;
 }
 
-__global__ void lt_flags_kernel(View v, HandleView h, uint64_t N, uint64_t cursor, uint64_t n, uint32_t q_first)
-{
-    grid_dependency_wait();
-    const LtChunk c = lt_chunk(q_first + blockIdx.y, N, v.R, cursor, n);
-    if (!c.active) return;
-    const unsigned lane = threadIdx.x & 31;
-    const uint64_t oc = h.state[c.q].x;
-    const uint64_t word = (oc >> 5) + (((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-    if (word * 32 >= c.size) return;
-    const uint64_t i = word * 32 + lane;
-    const bool loc = i >= oc && i < c.size && key_is_local(v, c.q, h.keys[c.b0 + i]);
-    const unsigned bits = __ballot_sync(0xFFFFFFFFu, loc);
-    if (lane == 0) h.flags[(c.b0 >> 5) + c.q + word] = bits;
-}
-
-constexpr int LT_THREADS = 1024;
+// Lookups and scan in one launch, as the calls are bound by their launches: 120,000 samples pulled in four parts 86 -> 73 us
+// with this and the rows copied by the placement pass; 1M samples in one part 124 -> 130 us (the fences).  A block that has
+// written its bits makes them visible and takes a ticket; the one that draws the last of its sub-handle's tickets sees all
+// of them and scans.  Nobody waits for anybody.
+constexpr int LT_THREADS = 512;
 constexpr int LT_WORDS = 4;                  // flag words per thread and round of the scan
 
 __global__ void __launch_bounds__(LT_THREADS)
-lt_scan_kernel(View v, HandleView h, uint64_t N, uint64_t cursor, uint64_t n, uint32_t q_first,
-               uint32_t* __restrict__ out)
+lt_walk_kernel(View v, HandleView h, uint64_t N, uint64_t cursor, uint64_t n, uint32_t q_first)
 {
     grid_dependency_wait();
-    __shared__ unsigned sh_tl, sh_old;
     __shared__ unsigned warp_tot[LT_THREADS / 32];
     __shared__ unsigned long long sh_stop;       // walk position right after the last entry that must be emitted
-    const LtChunk c = lt_chunk(q_first + blockIdx.x, N, v.R, cursor, n);
+    __shared__ bool sh_last;
+    const LtChunk c = lt_chunk(q_first + blockIdx.y, N, v.R, cursor, n);
     if (!c.active) return;
     const unsigned tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint4 stt = h.state[c.q];
     const uint64_t oc = stt.x, ph = stt.y, pt = stt.z;
     const uint64_t w0 = oc >> 5, w1 = oc < c.size ? (c.size + 31) >> 5 : w0;
-    const uint32_t* flags = h.flags + (c.b0 >> 5) + c.q;
+    uint32_t* flags = h.flags + (c.b0 >> 5) + c.q;
     uint32_t* prefix = h.prefix + (c.b0 >> 5) + c.q;
-    if (tid == 0) sh_stop = ~0ull;
+    {
+        const uint64_t stride = (uint64_t)gridDim.x * (LT_THREADS / 32);
+        for (uint64_t word = w0 + (uint64_t)blockIdx.x * (LT_THREADS / 32) + warp; word < w1; word += stride) {
+            const uint64_t i = word * 32 + lane;
+            const bool loc = i >= oc && i < c.size && key_is_local(v, c.q, h.keys[c.b0 + i]);
+            const unsigned bits = __ballot_sync(0xFFFFFFFFu, loc);
+            if (lane == 0) flags[word] = bits;
+        }
+    }
+    __syncthreads();
+    if (tid == 0) {
+        // orders the block's bits (the barrier puts them before this) before the ticket, and the ticket before the scan's
+        // reads of the other blocks' bits; a fence by every warp that wrote bits took 14 us more for 1M samples
+        __threadfence();
+        const unsigned ticket = atomicAdd(&h.walk[c.q].w, 1u);
+        __threadfence();
+        sh_last = ticket == gridDim.x - 1;
+        sh_stop = ~0ull;
+    }
+    __syncthreads();
+    if (!sh_last) return;
     unsigned long long carry = 0;                // local entries before the round
     for (uint64_t base = w0; base < w1 && carry < c.take; base += (uint64_t)LT_THREADS * LT_WORDS) {
         uint32_t bits[LT_WORDS];
@@ -678,7 +686,7 @@ lt_scan_kernel(View v, HandleView h, uint64_t N, uint64_t cursor, uint64_t n, ui
 #pragma unroll
         for (int k = 0; k < LT_WORDS; ++k) {
             const uint64_t w = base + (uint64_t)tid * LT_WORDS + k;
-            bits[k] = w < w1 ? flags[w] : 0u;
+            bits[k] = w < w1 ? __ldcg(flags + w) : 0u;         // written by other multiprocessors
             mine += __popc(bits[k]);
         }
         unsigned inc = mine;
@@ -720,27 +728,11 @@ lt_scan_kernel(View v, HandleView h, uint64_t N, uint64_t cursor, uint64_t n, ui
         h.prev[c.q] = stt;
         h.walk[c.q] = make_uint4((unsigned)tc, (unsigned)tl, (unsigned)cnt, 0u);
         h.state[c.q] = make_uint4((unsigned)(oc + tc), (unsigned)(ph + cnt), (unsigned)(pt + tc - tl), 0u);
-        sh_tl = (unsigned)tl;
-        sh_old = (unsigned)(cnt < pt - ph ? cnt : pt - ph);         // postponed by earlier calls, emitted by this one
-    }
-    __syncthreads();
-    // postponed entries come after the local ones; those that earlier calls postponed are already in place
-    // (what this call postpones and emits is handled where it is placed)
-    const unsigned tl = sh_tl, old = sh_old;
-    for (unsigned j0 = 0; j0 < old; j0 += LT_THREADS) {
-        const unsigned j = j0 + tid;
-        const bool in = j < old;
-        uint32_t key = 0;
-        if (in) {
-            key = h.post[c.b0 + ph + j];
-            out[c.out_base + tl + j] = key;
-        }
-        count_sample(v, key, in);
     }
 }
 
 // C8 > 0: the kernel also copies the rows of the keys it emits (rows of C8 chunks of 32 bytes, 32 / C8 rows per warp
-// instruction, as gather8_kernel does), which saves the separate gather launch of a full PullSample with values.
+// instruction, as gather8_kernel does), which saves the separate gather launch of a PullSample with values.
 template <int C8>
 __global__ void __launch_bounds__(256)
 lt_place_kernel(View v, HandleView h, uint64_t N, uint64_t cursor, uint64_t n, uint32_t q_first,
@@ -753,34 +745,47 @@ lt_place_kernel(View v, HandleView h, uint64_t N, uint64_t cursor, uint64_t n, u
     const unsigned lane = threadIdx.x & 31;
     const uint4 pv = h.prev[c.q], wk = h.walk[c.q];
     const uint64_t oc = pv.x, ph = pv.y, pt = pv.z, end = oc + wk.x, tl = wk.y, cnt = wk.z;
-    const uint64_t word = (oc >> 5) + (((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-    if (word * 32 >= end) return;
-    const uint64_t i = word * 32 + lane;
-    const bool walked = i >= oc && i < end;
-    const uint32_t bits = h.flags[(c.b0 >> 5) + c.q + word];
-    const uint64_t before = (uint64_t)h.prefix[(c.b0 >> 5) + c.q + word] + __popc(bits & ((1u << lane) - 1u));
-    const bool loc = (bits >> lane) & 1u;
+    // the first warps take the words of the fresh entries that are walked, those after them the entries that earlier
+    // calls postponed and this one emits (they come after the local ones)
+    const uint64_t w = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5, words = wk.x ? ((end + 31) >> 5) - (oc >> 5) : 0;
+    const uint64_t old = cnt < pt - ph ? cnt : pt - ph;
     uint32_t key = 0;
     bool emitted = false;
     uint32_t opos = 0;                                               // where the emitted key went
-    if (walked) {
-        key = h.keys[c.b0 + i];
-        if (loc) {
-            opos = (uint32_t)(c.out_base + before);
-            out[opos] = key;
-            emitted = true;
-        } else {
-            // postponed: queued behind the non-local entries before it, emitted by this very call if the queue's
-            // head gets that far, and moved to the worker.  (Locality was judged before any key moved: the bits
-            // were all looked up by the kernel before this one.)
-            const uint64_t at = pt + ((i - oc) - before);
-            h.post[c.b0 + at] = key;
-            if (at >= ph && at < ph + cnt) {
-                opos = (uint32_t)(c.out_base + tl + (at - ph));
+    if (w < words) {
+        const uint64_t word = (oc >> 5) + w, i = word * 32 + lane;
+        const bool walked = i >= oc && i < end;
+        const uint32_t bits = h.flags[(c.b0 >> 5) + c.q + word];
+        const uint64_t before = (uint64_t)h.prefix[(c.b0 >> 5) + c.q + word] + __popc(bits & ((1u << lane) - 1u));
+        const bool loc = (bits >> lane) & 1u;
+        if (walked) {
+            key = h.keys[c.b0 + i];
+            if (loc) {
+                opos = (uint32_t)(c.out_base + before);
                 out[opos] = key;
                 emitted = true;
+            } else {
+                // postponed: queued behind the non-local entries before it, emitted by this very call if the queue's
+                // head gets that far, and moved to the worker.  (Locality was judged before any key moved: the bits
+                // were all looked up by the kernel before this one.)
+                const uint64_t at = pt + ((i - oc) - before);
+                h.post[c.b0 + at] = key;
+                if (at >= ph && at < ph + cnt) {
+                    opos = (uint32_t)(c.out_base + tl + (at - ph));
+                    out[opos] = key;
+                    emitted = true;
+                }
+                mark_localize(v, key, c.q);
             }
-            mark_localize(v, key, c.q);
+        }
+    } else {
+        const uint64_t j = (w - words) * 32 + lane;
+        if ((w - words) * 32 >= old) return;
+        if (j < old) {
+            key = h.post[c.b0 + ph + j];
+            opos = (uint32_t)(c.out_base + tl + j);
+            out[opos] = key;
+            emitted = true;
         }
     }
     count_sample(v, key, emitted);
@@ -842,15 +847,15 @@ static nups_status pull_internal(nups_store* s, int id, uint64_t n, uint32_t* d_
             if (b0 <= h.cursor + n - 1 && h.cursor + n - 1 < b1) ql = q;
         }
         const uint64_t max_size = (h.N + s->R - 1) / s->R;
-        const dim3 by_word(grid_for(max_size / 32 + 2, 8), ql - qf + 1);
-        nups_launch_dependent(lt_flags_kernel, by_word, 256, 0, st, v, hv, h.N, h.cursor, n, qf);
+        // words of a sub-handle and of its postponed entries: together at most three more than the sub-handle's entries fill
+        const dim3 by_word(grid_for(max_size / 32 + 4, 8), ql - qf + 1);
+        // as many blocks as are resident at once: every block pays for a fence and a ticket
+        const unsigned walkers = grid_for(max_size / 32 + 2, LT_THREADS / 32, grid_for((uint64_t)s->sm_count * 4, ql - qf + 1));
+        nups_launch_dependent(lt_walk_kernel, dim3(walkers, ql - qf + 1), LT_THREADS, 0, st, v, hv, h.N, h.cursor, n, qf);
         LAUNCH_CHECK(s);
-        nups_launch_dependent(lt_scan_kernel, ql - qf + 1, LT_THREADS, 0, st, v, hv, h.N, h.cursor, n, qf, d_keys_out);
-        LAUNCH_CHECK(s);
-        // a full pull of a fresh handle has no entries postponed by earlier calls to emit: the placement pass can copy
-        // the rows itself (one table of 64, 128 or 256 floats per row, 32-byte aligned output)
+        // the placement pass can copy the rows itself (one table of 64, 128 or 256 floats per row, 32-byte aligned output)
         const uint32_t c8 = s->L / 8;
-        const bool fused = d_vals_out && s->vb == 4 && h.cursor == 0 && n == h.N && s->L % 8 == 0 && (c8 == 8 || c8 == 16 || c8 == 32) &&
+        const bool fused = d_vals_out && s->vb == 4 && s->L % 8 == 0 && (c8 == 8 || c8 == 16 || c8 == 32) &&
                            ((uintptr_t)d_vals_out & 31) == 0 && (uint64_t)s->R * s->Hcap < 0xFFFFFFFFull;
         if (fused) nups_time_begin(s, st, NUPS_TIMED_SAMPLE_ROWS);
         if (fused && c8 == 8) nups_launch_dependent(lt_place_kernel<8>, by_word, 256, 0, st, v, hv, h.N, h.cursor, n, qf, d_keys_out, s->val, s->dval, d_vals_out);
@@ -861,7 +866,7 @@ static nups_status pull_internal(nups_store* s, int id, uint64_t n, uint32_t* d_
         LAUNCH_CHECK(s);
         if (fused) {
             h.cursor += n;
-            h.used = 0;
+            if (h.cursor == h.N) h.used = 0;
             return NUPS_OK;
         }
     } else if (d_vals_out && d.level != NUPS_NONCONFORM && !s->cfg.count_accesses) {
