@@ -630,6 +630,29 @@ struct PushPair {
     float* slab;           // replica slabs
 };
 
+// What a lane takes of a row at a time: 16 bytes of 4-byte values, one reduction for all four; single 8-byte values, for which
+// there is no wider reduction, so that the lanes of one reduction touch consecutive values (two per lane, 16 bytes apart from
+// lane to lane, use half of every sector: 300,000 rows of 128 values 180 -> 135 us).
+template <bool F64>
+struct PushElement {
+    using T = float4;
+    static __device__ __forceinline__ T zero() { return make_float4(0.f, 0.f, 0.f, 0.f); }
+    static __device__ __forceinline__ T load(const float4* p, uint64_t i) { return ld_stream_v4(p + i); }
+    static __device__ __forceinline__ T add(T a, T b) { return add4(a, b); }
+    static __device__ __forceinline__ void reduce(float* base, uint64_t i, T x) { red_add_v4(base + 4 * i, x); }
+};
+template <>
+struct PushElement<true> {
+    using T = double;
+    static __device__ __forceinline__ T zero() { return 0.0; }
+    static __device__ __forceinline__ T load(const float4* p, uint64_t i) { return __ldcs(reinterpret_cast<const double*>(p) + i); }
+    static __device__ __forceinline__ T add(T a, T b) { return a + b; }
+    static __device__ __forceinline__ void reduce(float* base, uint64_t i, T x)
+    {
+        asm volatile("red.global.add.f64 [%0], %1;" ::"l"(reinterpret_cast<double*>(base) + i), "d"(x) : "memory");
+    }
+};
+
 // TIER = the block keeps shared-memory accumulators for the hottest replica slots (slot < tier_rows)
 // of ONE worker (block b serves worker b mod R and visits only that worker's share of the windows);
 // updates to those slots are added in shared memory and reach the worker's replica once, when the
@@ -648,7 +671,8 @@ push_atomic_kernel(View v, const uint32_t* __restrict__ keys, uint64_t n, PushPa
     grid_dependency_wait();
     extern __shared__ __align__(16) float tier_mem[];                  // TIER: [tier_rows][L] sums, then touched bits
     const unsigned lane = threadIdx.x & 31;
-    const uint32_t L4 = v.L4;
+    using E = PushElement<F64>;
+    const uint32_t L4 = v.L4, LE = F64 ? 2 * L4 : L4;                  // a row's length in 16-byte chunks and in elements
     const uint32_t R = v.R;
     unsigned* touched = reinterpret_cast<unsigned*>(tier_mem + (size_t)tier_rows * L4 * 4);
     unsigned* tags = touched + (tier_rows + 31) / 32;                  // TIER == 2: key that owns each accumulator
@@ -754,30 +778,67 @@ push_atomic_kernel(View v, const uint32_t* __restrict__ keys, uint64_t n, PushPa
                 de[u4] = __shfl_sync(0xFFFFFFFFu, dest, src[u4] < 0 ? 0 : src[u4]);
                 tr[u4] = TIER ? __shfl_sync(0xFFFFFFFFu, tier, src[u4] < 0 ? 0 : src[u4]) : -1;
             }
-            for (uint32_t c = lane; c < L4; c += 32) {
-                float4 a[PUSH_UNROLL], b[PUSH_UNROLL];
+            if constexpr (F64) {
+                // the two rows one after the other in one run of lanes: a row that does not fill its last 32 lanes leaves
+                // them to the next one
+                static_assert(PUSH_UNROLL == 2, "two rows share a run of lanes");
+                const uint32_t both = src[1] >= 0 ? 2 * LE : LE;
+                for (uint32_t e0 = lane; e0 < both; e0 += 64) {
+                    typename E::T a[2], b[2];
+                    uint32_t c[2];
+                    bool second[2];
+#pragma unroll
+                    for (int k = 0; k < 2; ++k) {
+                        second[k] = e0 + 32 * k >= LE;
+                        c[k] = e0 + 32 * k - (second[k] ? LE : 0u);
+                        if (e0 + 32 * k < both) {
+                            const uint64_t in_off = (base + (second[k] ? src[1] : src[0])) * LE + c[k];
+                            a[k] = E::load(A.delta, in_off);
+                            if (TWO) b[k] = E::load(B.delta, in_off);
+                        }
+                    }
+#pragma unroll
+                    for (int k = 0; k < 2; ++k) {
+                        if (e0 + 32 * k < both) {
+                            const unsigned long long d = second[k] ? de[1] : de[0];
+                            const bool h = HOT && (d & 1ull);
+                            const uint64_t off = (d >> 3) * 2 + c[k];
+                            E::reduce(h ? A.slab : A.table, off, a[k]);
+                            if (TWO) E::reduce(h ? B.slab : B.table, off, b[k]);
+                        }
+                    }
+                }
+                continue;
+            }
+            for (uint32_t c = lane; c < LE; c += 32) {
+                typename E::T a[PUSH_UNROLL], b[PUSH_UNROLL];
 #pragma unroll
                 for (int u4 = 0; u4 < PUSH_UNROLL; ++u4) {
                     if (src[u4] >= 0) {
-                        const uint64_t in_off = (base + src[u4]) * L4 + c;
-                        a[u4] = ld_stream_v4(A.delta + in_off);
-                        if (TWO) b[u4] = ld_stream_v4(B.delta + in_off);
+                        const uint64_t in_off = (base + src[u4]) * LE + c;
+                        a[u4] = E::load(A.delta, in_off);
+                        if (TWO) b[u4] = E::load(B.delta, in_off);
                     }
                 }
 #pragma unroll
                 for (int u4 = 0; u4 < PUSH_UNROLL; ++u4) {
                     if (src[u4] >= 0) {
-                        if (TIER && tr[u4] >= 0) {
-                            // accumulator rows are stored component by component, [4][L4], so that the 32
-                            // lanes of one addition fall into 32 different banks
-                            float* t = tier_mem + (size_t)tr[u4] * L4 * 4 + c;
-                            atomicAdd(t, a[u4].x); atomicAdd(t + L4, a[u4].y); atomicAdd(t + 2 * L4, a[u4].z);
-                            atomicAdd(t + 3 * L4, a[u4].w);
-                        } else {
+                        bool in_tier = false;
+                        if constexpr (TIER != 0) {
+                            in_tier = tr[u4] >= 0;
+                            if (in_tier) {
+                                // accumulator rows are stored component by component, [4][L4], so that the 32
+                                // lanes of one addition fall into 32 different banks
+                                float* t = tier_mem + (size_t)tr[u4] * L4 * 4 + c;
+                                atomicAdd(t, a[u4].x); atomicAdd(t + L4, a[u4].y); atomicAdd(t + 2 * L4, a[u4].z);
+                                atomicAdd(t + 3 * L4, a[u4].w);
+                            }
+                        }
+                        if (!in_tier) {
                             const bool h = HOT && (de[u4] & 1ull);
-                            const uint64_t off = (de[u4] >> 3) * 4 + (uint64_t)c * 4;
-                            red_add_chunk<F64>((h ? A.slab : A.table) + off, a[u4]);
-                            if (TWO) red_add_chunk<F64>((h ? B.slab : B.table) + off, b[u4]);
+                            const uint64_t off = (de[u4] >> 3) * (F64 ? 2 : 1) + c;
+                            E::reduce(h ? A.slab : A.table, off, a[u4]);
+                            if (TWO) E::reduce(h ? B.slab : B.table, off, b[u4]);
                         }
                     }
                 }
@@ -797,12 +858,12 @@ push_atomic_kernel(View v, const uint32_t* __restrict__ keys, uint64_t n, PushPa
             const unsigned long long de = __shfl_sync(0xFFFFFFFFu, dest, ld);
             const int tr = TIER ? __shfl_sync(0xFFFFFFFFu, tier, ld) : -1;
             const bool h = HOT && (de & 1ull);
-            for (uint32_t c = lane; c < L4; c += 32) {
-                float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
+            for (uint32_t c = lane; c < LE; c += 32) {
+                typename E::T a = E::zero(), b = a;
                 unsigned mm = members;
                 while (mm) {
                     int m[PUSH_UNROLL];
-                    float4 x[PUSH_UNROLL], y[PUSH_UNROLL];
+                    typename E::T x[PUSH_UNROLL], y[PUSH_UNROLL];
 #pragma unroll
                     for (int u4 = 0; u4 < PUSH_UNROLL; ++u4) {
                         m[u4] = mm ? __ffs(mm) - 1 : -1;
@@ -811,26 +872,31 @@ push_atomic_kernel(View v, const uint32_t* __restrict__ keys, uint64_t n, PushPa
 #pragma unroll
                     for (int u4 = 0; u4 < PUSH_UNROLL; ++u4) {
                         if (m[u4] >= 0) {
-                            const uint64_t in_off = (base + m[u4]) * L4 + c;
-                            x[u4] = ld_stream_v4(A.delta + in_off);
-                            if (TWO) y[u4] = ld_stream_v4(B.delta + in_off);
+                            const uint64_t in_off = (base + m[u4]) * LE + c;
+                            x[u4] = E::load(A.delta, in_off);
+                            if (TWO) y[u4] = E::load(B.delta, in_off);
                         }
                     }
 #pragma unroll
                     for (int u4 = 0; u4 < PUSH_UNROLL; ++u4) {
                         if (m[u4] >= 0) {
-                            a = add_chunk<F64>(a, x[u4]);
-                            if (TWO) b = add_chunk<F64>(b, y[u4]);
+                            a = E::add(a, x[u4]);
+                            if (TWO) b = E::add(b, y[u4]);
                         }
                     }
                 }
-                if (TIER && tr >= 0) {
-                    float* t = tier_mem + (size_t)tr * L4 * 4 + c;
-                    atomicAdd(t, a.x); atomicAdd(t + L4, a.y); atomicAdd(t + 2 * L4, a.z); atomicAdd(t + 3 * L4, a.w);
-                } else {
-                    const uint64_t off = (de >> 3) * 4 + (uint64_t)c * 4;
-                    red_add_chunk<F64>((h ? A.slab : A.table) + off, a);
-                    if (TWO) red_add_chunk<F64>((h ? B.slab : B.table) + off, b);
+                bool in_tier = false;
+                if constexpr (TIER != 0) {
+                    in_tier = tr >= 0;
+                    if (in_tier) {
+                        float* t = tier_mem + (size_t)tr * L4 * 4 + c;
+                        atomicAdd(t, a.x); atomicAdd(t + L4, a.y); atomicAdd(t + 2 * L4, a.z); atomicAdd(t + 3 * L4, a.w);
+                    }
+                }
+                if (!in_tier) {
+                    const uint64_t off = (de >> 3) * (F64 ? 2 : 1) + c;
+                    E::reduce(h ? A.slab : A.table, off, a);
+                    if (TWO) E::reduce(h ? B.slab : B.table, off, b);
                 }
             }
             if (TIER && tr >= 0 && lane == 0 && !((touched[tr >> 5] >> (tr & 31)) & 1u))
