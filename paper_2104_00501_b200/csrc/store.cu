@@ -370,12 +370,14 @@ struct TablePair {
 template <bool HOT, bool TWO, bool F64>
 __global__ void __launch_bounds__(256, 4)
 gather_kernel(View v, const uint32_t* __restrict__ keys, uint64_t n, TablePair A, TablePair B, int map,
-              uint64_t map_base, uint64_t map_total, int do_count, uint32_t* __restrict__ keys_copy)
+              uint64_t map_base, uint64_t map_total, int do_count, uint32_t* __restrict__ keys_copy, uint32_t parts)
 {
     grid_dependency_wait();
     const unsigned lane = threadIdx.x & 31;
-    const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+    const uint64_t team = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5, warp = team / parts;
+    const uint32_t part = (uint32_t)(team - warp * parts);         // this warp's share of the window's rows
+    const uint64_t nwarps = (((uint64_t)gridDim.x * blockDim.x) >> 5) / parts;
+    if (warp >= nwarps) return;
     const uint32_t L4 = v.L4;
     // Lookups run ahead of the copies: while window w is copied, the key of window w + 2 and the
     // hot-bit word of window w + 1 are already on their way.
@@ -393,8 +395,8 @@ gather_kernel(View v, const uint32_t* __restrict__ keys, uint64_t n, TablePair A
         bits_a = (HOT && key_a < v.num_keys) ? __ldg(v.hot_bits + (key_a >> 5)) : 0u;
         key_b = base + 2 * stride + lane < n ? __ldg(keys + base + 2 * stride + lane) : 0u;
         const bool valid = in && key < v.num_keys;
-        if (in && !valid) flag_bad_key(v);
-        if (keys_copy && in) keys_copy[i] = key;                   // PullSample hands the keys out as well
+        if (in && !valid && part == 0) flag_bad_key(v);
+        if (keys_copy && in && part == 0) keys_copy[i] = key;                   // PullSample hands the keys out as well
         unsigned long long src = valid ? (unsigned long long)key * L4 : NO_ROW;   // NO_ROW: zero-filled output
         unsigned long long pend = NO_ROW;
         if (HOT && valid && ((bits >> (key & 31)) & 1u)) {
@@ -403,7 +405,7 @@ gather_kernel(View v, const uint32_t* __restrict__ keys, uint64_t n, TablePair A
             const uint32_t q = map == 0 ? worker_of_item(idx, map_total, v.R) : chunk_of_pos(idx, map_total, v.R);
             pend = ((unsigned long long)q * v.Hcap + slot) * L4;
         }
-        if (do_count && v.count) {
+        if (do_count && v.count && part == 0) {
             if (valid) atomicAdd(v.cnt + key, 1ull);
             unsigned hot_m = __ballot_sync(0xFFFFFFFFu, valid && pend != NO_ROW);
             unsigned cold_m = __ballot_sync(0xFFFFFFFFu, valid && pend == NO_ROW);
@@ -412,8 +414,8 @@ gather_kernel(View v, const uint32_t* __restrict__ keys, uint64_t n, TablePair A
                 if (cold_m) atomicAdd(&v.st->cold_hits, (unsigned long long)__popc(cold_m));
             }
         }
-        const int rows = (int)min((uint64_t)32, n - base);
-        for (int r = 0; r < rows; r += GATHER_UNROLL) {
+        const int rows = (int)min((uint64_t)32, n - base), share = 32 / (int)parts;
+        for (int r = (int)part * share; r < min(rows, ((int)part + 1) * share); r += GATHER_UNROLL) {
             unsigned long long so[GATHER_UNROLL], po[GATHER_UNROLL];
 #pragma unroll
             for (int u = 0; u < GATHER_UNROLL; ++u) {
@@ -463,15 +465,17 @@ template <bool HOT, int C8>
 __global__ void __launch_bounds__(256, 4)
 gather8_kernel(View v, const uint32_t* __restrict__ keys, uint64_t n, const float* __restrict__ table,
                const float* slab, float* __restrict__ out, int map, uint64_t map_base, uint64_t map_total, int do_count,
-               uint32_t* __restrict__ keys_copy)
+               uint32_t* __restrict__ keys_copy, uint32_t parts)
 {
     grid_dependency_wait();
     constexpr int RPI = 32 / C8;                       // rows per warp instruction
     constexpr int UNR = 2;                             // instructions in flight
     const unsigned lane = threadIdx.x & 31;
     const unsigned sub = lane / C8, c = lane % C8;     // which of the instruction's rows, which chunk of it
-    const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+    const uint64_t team = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5, warp = team / parts;
+    const uint32_t part = (uint32_t)(team - warp * parts);         // this warp's share of the window's rows
+    const uint64_t nwarps = (((uint64_t)gridDim.x * blockDim.x) >> 5) / parts;
+    if (warp >= nwarps) return;
     const uint64_t L = (uint64_t)v.L4 * 4;
     const uint64_t stride = nwarps * 32;
     uint64_t base = warp * 32;
@@ -488,8 +492,8 @@ gather8_kernel(View v, const uint32_t* __restrict__ keys, uint64_t n, const floa
         bits_a = (HOT && key_a < v.num_keys) ? __ldg(v.hot_bits + (key_a >> 5)) : 0u;
         key_b = base + 2 * stride + lane < end ? __ldg(keys + base + 2 * stride + lane) : 0u;
         const bool valid = in && key < v.num_keys;
-        if (in && !valid) flag_bad_key(v);
-        if (keys_copy && in) keys_copy[i] = key;                   // PullSample hands the keys out as well
+        if (in && !valid && part == 0) flag_bad_key(v);
+        if (keys_copy && in && part == 0) keys_copy[i] = key;                   // PullSample hands the keys out as well
         // row numbers instead of offsets: one 32-bit shuffle each; 0xFFFFFFFF = no such row
         uint32_t src = valid ? key : 0xFFFFFFFFu;
         uint32_t pend = 0xFFFFFFFFu;                    // replica row (worker * Hcap + slot) of a replicated key
@@ -499,7 +503,7 @@ gather8_kernel(View v, const uint32_t* __restrict__ keys, uint64_t n, const floa
             const uint32_t q = map == 0 ? worker_of_item(idx, map_total, v.R) : chunk_of_pos(idx, map_total, v.R);
             pend = q * (uint32_t)v.Hcap + slot;
         }
-        if (do_count && v.count) {
+        if (do_count && v.count && part == 0) {
             if (valid) atomicAdd(v.cnt + key, 1ull);
             unsigned hot_m = __ballot_sync(0xFFFFFFFFu, valid && pend != 0xFFFFFFFFu);
             unsigned cold_m = __ballot_sync(0xFFFFFFFFu, valid && pend == 0xFFFFFFFFu);
@@ -508,8 +512,8 @@ gather8_kernel(View v, const uint32_t* __restrict__ keys, uint64_t n, const floa
                 if (cold_m) atomicAdd(&v.st->cold_hits, (unsigned long long)__popc(cold_m));
             }
         }
-        const int rows = (int)min((uint64_t)32, end - base);
-        for (int r0 = 0; r0 < rows; r0 += UNR * RPI) {
+        const int share = 32 / (int)parts, rows = (int)min((uint64_t)((part + 1) * share), end - base);
+        for (int r0 = (int)part * share; r0 < rows; r0 += UNR * RPI) {
             uint32_t so[UNR], po[UNR];
             F8 a[UNR];
 #pragma unroll
@@ -543,6 +547,18 @@ gather8_kernel(View v, const uint32_t* __restrict__ keys, uint64_t n, const floa
     }
 }
 
+// Into how many warps (a power of two, at most `most`) the rows of a window of 32 are divided, so that up to `resident` warps
+// have work.  A warp takes its rows a few at a time, one memory latency after the other, so the windows of a small call would
+// leave most multiprocessors idle while a few warps wait eight times in a row; every warp of a window repeats its lookups.
+// Measured: pulling 50,000 rows of 100 floats 13.7 -> 9.9 us, pushing 5,000 10.3 -> 6.8 us, a round of pull and push over two
+// tables with 20,000 rows 43 -> 30 us.
+static uint32_t window_parts(uint64_t rows, uint64_t resident, uint32_t most)
+{
+    uint32_t parts = 1;
+    while (parts < most && (rows + 31) / 32 * (2 * parts) <= resident) parts *= 2;
+    return parts;
+}
+
 nups_status nups_gather_internal(nups_store* s, const uint32_t* d_keys, uint64_t n, float* d_out_val,
                                  float* d_out_acc, int worker_map, uint64_t map_base, uint64_t map_total,
                                  int do_count, cudaStream_t st, uint32_t* d_keys_copy)
@@ -553,7 +569,9 @@ nups_status nups_gather_internal(nups_store* s, const uint32_t* d_keys, uint64_t
     TablePair C = {(const float4*)s->acc, (const float4*)s->dacc, (float4*)d_out_acc};
     const bool two = d_out_val && d_out_acc;
     TablePair A = d_out_val ? V : C, B = C;
-    unsigned grid = grid_for(n, 32 * 8, (unsigned)s->sm_count * 4);     // 4 resident blocks per SM, grid-stride
+    // 4 resident blocks per SM, grid-stride.  Fewer rows than keep them all busy: several warps share a window of 32 rows.
+    const uint32_t parts = window_parts(n, (uint64_t)s->sm_count * 4 * 8, 8);
+    unsigned grid = grid_for(n * parts, 32 * 8, (unsigned)s->sm_count * 4);
     // one table, rows of 8, 16 or 32 chunks of 32 bytes, everything 32-byte aligned, some keys replicated: the
     // 256-bit variant.  (Measured on 1M-key pulls of 128-float rows: with a hot tier 152 vs 163 us at Zipf 1.0 and
     // 20-25 % faster when keys repeat as under sample reuse; without a hot tier, where every row comes from DRAM,
@@ -567,7 +585,7 @@ nups_status nups_gather_internal(nups_store* s, const uint32_t* d_keys, uint64_t
         nups_time_begin(s, st, worker_map == 1 ? NUPS_TIMED_SAMPLE_ROWS : NUPS_TIMED_PULL);
 #define NUPS_G8(C8_)                                                                                                     \
         nups_launch_dependent(gather8_kernel<true, C8_>, grid, 256, 0, st, v, d_keys, n, table, slab, out1, worker_map, map_base, map_total, \
-                                                        do_count, d_keys_copy)
+                                                        do_count, d_keys_copy, parts)
         if (c8 == 8) NUPS_G8(8);
         else if (c8 == 16) NUPS_G8(16);
         else NUPS_G8(32);
@@ -579,7 +597,7 @@ nups_status nups_gather_internal(nups_store* s, const uint32_t* d_keys, uint64_t
     nups_time_begin(s, st, worker_map == 1 ? NUPS_TIMED_SAMPLE_ROWS : NUPS_TIMED_PULL);
 #define NUPS_GATHER(HOT_, TWO_, F64_)                                                                                  \
     nups_launch_dependent(gather_kernel<HOT_, TWO_, F64_>, grid, 256, 0, st, v, d_keys, n, A, B, worker_map, map_base, map_total, do_count, \
-                                                          d_keys_copy)
+                                                          d_keys_copy, parts)
     if (s->vb == 8) {                        // only replica reads add; rows without a replica are copied whatever they hold
         if (s->H) { if (two) NUPS_GATHER(true, true, true); else NUPS_GATHER(true, false, true); }
         else { if (two) NUPS_GATHER(false, true, false); else NUPS_GATHER(false, false, false); }
@@ -663,10 +681,11 @@ struct PushElement<true> {
 // takes that key's updates until the block ends (other keys that map there go straight to their rows).  Frequent
 // keys show up early and often, so they take most accumulators, and a skewed batch stops queueing at a few L2
 // addresses even when its frequent keys were never marked for replication.
-template <bool HOT, bool TWO, int TIER, bool F64>
+// PARTS = several warps share a window of rows (see window_parts); the kernel of the largest calls does without the registers.
+template <bool HOT, bool TWO, int TIER, bool F64, bool PARTS>
 __global__ void __launch_bounds__(PUSH_THREADS, TWO ? PUSH_BLOCKS - 1 : PUSH_BLOCKS)
 push_atomic_kernel(View v, const uint32_t* __restrict__ keys, uint64_t n, PushPair A, PushPair B, uint64_t n_items,
-                   uint32_t rows_per_item, uint32_t tier_rows)
+                   uint32_t rows_per_item, uint32_t tier_rows, uint32_t parts)
 {
     grid_dependency_wait();
     extern __shared__ __align__(16) float tier_mem[];                  // TIER: [tier_rows][L] sums, then touched bits
@@ -691,9 +710,10 @@ push_atomic_kernel(View v, const uint32_t* __restrict__ keys, uint64_t n, PushPa
     const uint64_t W = (n + 31) / 32;
     const uint64_t per = (W + R - 1) / R;
     const uint32_t my_q = TIER == 1 ? blockIdx.x % R : 0u;
-    const uint64_t warp = TIER == 1 ? ((uint64_t)(blockIdx.x / R) * blockDim.x + threadIdx.x) >> 5
-                               : ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const uint64_t nwarps = TIER == 1 ? ((uint64_t)(gridDim.x / R) * blockDim.x) >> 5 : ((uint64_t)gridDim.x * blockDim.x) >> 5;
+    const uint64_t team = ((uint64_t)(TIER == 1 ? blockIdx.x / R : blockIdx.x) * blockDim.x + threadIdx.x) >> 5, warp = PARTS ? team / parts : team;
+    const uint32_t part = PARTS ? (uint32_t)(team - warp * parts) : 0u;            // this warp's share of the window's destinations
+    const uint64_t teams = ((uint64_t)(TIER == 1 ? gridDim.x / R : gridDim.x) * blockDim.x) >> 5, nwarps = PARTS ? teams / parts : teams;
+    const unsigned share = !PARTS ? 0xFFFFFFFFu : (parts == 1 ? 0xFFFFFFFFu : parts == 2 ? 0x55555555u : parts == 4 ? 0x11111111u : 0x01010101u) << part;
     const uint64_t slots = TIER == 1 ? per : per * R;
     auto window_of = [&](uint64_t u) -> uint64_t {
         if (u >= slots) return W;
@@ -720,7 +740,7 @@ push_atomic_kernel(View v, const uint32_t* __restrict__ keys, uint64_t n, PushPa
         const uint64_t i = base + lane;
         const bool in = i < n;
         const bool valid = in && key < v.num_keys;
-        if (in && !valid) flag_bad_key(v);
+        if (in && !valid && part == 0) flag_bad_key(v);
         // destination: row offset in floats, lowest bit set when it lies in the replica slab
         unsigned long long dest = NO_ROW - lane;          // invalid rows: a value no other lane has
         bool hot = false;
@@ -747,7 +767,7 @@ push_atomic_kernel(View v, const uint32_t* __restrict__ keys, uint64_t n, PushPa
                 if (owner == key) tier = (int)at;
             }
         }
-        if (v.count) {
+        if (v.count && part == 0) {
             if (valid) atomicAdd(v.cnt + key, 1ull);
             unsigned hot_m = __ballot_sync(0xFFFFFFFFu, valid && hot);
             unsigned cold_m = __ballot_sync(0xFFFFFFFFu, valid && !hot);
@@ -764,8 +784,8 @@ push_atomic_kernel(View v, const uint32_t* __restrict__ keys, uint64_t n, PushPa
             uint32_t* flag = v.dirty + hrow;          // replica row index = q * Hcap + slot
             if (*flag == 0u) *flag = 1u;
         }
-        unsigned singles = __ballot_sync(0xFFFFFFFFu, leader && __popc(grp) == 1);
-        unsigned multis = __ballot_sync(0xFFFFFFFFu, leader && __popc(grp) > 1);
+        unsigned singles = __ballot_sync(0xFFFFFFFFu, leader && __popc(grp) == 1) & share;
+        unsigned multis = __ballot_sync(0xFFFFFFFFu, leader && __popc(grp) > 1) & share;
 
         // rows that are alone in their window: PUSH_UNROLL at a time
         while (singles) {
@@ -1370,7 +1390,7 @@ nups_status nups_push_with_scratch(nups_store* s, const uint32_t* d_keys, uint64
     uint64_t n_items = n / rows_per_item;
     if (!s->cfg.deterministic) {
         const bool two = d_dval && d_dacc;
-        unsigned grid = grid_for(n, PUSH_THREADS, (unsigned)s->sm_count * (two ? PUSH_BLOCKS - 1 : PUSH_BLOCKS));  // resident at once, grid-stride
+        const unsigned blocks = (unsigned)s->sm_count * (two ? PUSH_BLOCKS - 1 : PUSH_BLOCKS);
         PushPair V = {(const float4*)d_dval, s->val, s->dval};
         PushPair C = {(const float4*)d_dacc, s->acc, s->dacc};
         PushPair A = d_dval ? V : C, B = C;
@@ -1378,6 +1398,9 @@ nups_status nups_push_with_scratch(nups_store* s, const uint32_t* d_keys, uint64
         uint32_t tier_rows = 0;
         size_t tier_bytes = 0;
         const bool cache = !s->H && !two && n >= 32768 && s->vb == 4;  // no replicated keys: accumulators as a row cache
+        // (with the row cache, more blocks cost more accumulators to fill and to hand over than they save: 40,000 rows 17 -> 19 us)
+        const uint32_t parts = cache ? 1 : window_parts(n, (uint64_t)blocks * (PUSH_THREADS / 32), 8);
+        unsigned grid = grid_for(n * parts, PUSH_THREADS, blocks);                 // resident at once, grid-stride
         if ((s->H && !two && rows_per_item == 1 && grid >= s->R && n >= 32768 && s->vb == 4) || cache) {
             const size_t row_bytes = (size_t)s->L * 4;
             size_t budget = (size_t)(192 / PUSH_BLOCKS) * 1024;                 // the blocks of a multiprocessor share 192 KB
@@ -1388,24 +1411,26 @@ nups_status nups_push_with_scratch(nups_store* s, const uint32_t* d_keys, uint64
             if (!cache && tier_rows > s->H) tier_rows = (uint32_t)s->H;
             tier_bytes = tier_rows * row_bytes + ((tier_rows + 31) / 32) * 4 + (cache ? tier_rows * 4 : 0);
             if (tier_rows && !s->push_smem_opted) {
-                CK(cudaFuncSetAttribute(push_atomic_kernel<true, false, 1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                CK(cudaFuncSetAttribute(push_atomic_kernel<true, false, 1, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         (int)(budget + 2048)));
-                CK(cudaFuncSetAttribute(push_atomic_kernel<false, false, 2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                CK(cudaFuncSetAttribute(push_atomic_kernel<true, false, 1, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)(budget + 2048)));
+                CK(cudaFuncSetAttribute(push_atomic_kernel<false, false, 2, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         (int)(budget + 2048)));
                 s->push_smem_opted = true;
             }
         }
         nups_time_begin(s, st, NUPS_TIMED_PUSH);
         if (tier_rows && cache) {
-            nups_launch_dependent(push_atomic_kernel<false, false, 2, false>, grid, PUSH_THREADS, tier_bytes, st, v, d_keys, n, A, B, n_items, rows_per_item,
-                                                                             tier_rows);
+            nups_launch_dependent(push_atomic_kernel<false, false, 2, false, false>, grid, PUSH_THREADS, tier_bytes, st, v, d_keys, n, A, B, n_items, rows_per_item,
+                                                                             tier_rows, parts);
         } else if (tier_rows) {
             grid = grid / s->R * s->R;              // every worker gets the same number of blocks
-            nups_launch_dependent(push_atomic_kernel<true, false, 1, false>, grid, PUSH_THREADS, tier_bytes, st, v, d_keys, n, A, B, n_items, rows_per_item,
-                                                                             tier_rows);
+            nups_launch_dependent(parts > 1 ? push_atomic_kernel<true, false, 1, false, true> : push_atomic_kernel<true, false, 1, false, false>, grid, PUSH_THREADS, tier_bytes, st, v, d_keys, n, A, B, n_items, rows_per_item,
+                                                                             tier_rows, parts);
         } else {
 #define NUPS_PUSH0(HOT_, TWO_, F64_) \
-    nups_launch_dependent(push_atomic_kernel<HOT_, TWO_, 0, F64_>, grid, PUSH_THREADS, 0, st, v, d_keys, n, A, B, n_items, rows_per_item, 0)
+    nups_launch_dependent(push_atomic_kernel<HOT_, TWO_, 0, F64_, true>, grid, PUSH_THREADS, 0, st, v, d_keys, n, A, B, n_items, rows_per_item, 0, parts)
             if (s->vb == 8) {
                 if (s->H) { if (two) NUPS_PUSH0(true, true, true); else NUPS_PUSH0(true, false, true); }
                 else { if (two) NUPS_PUSH0(false, true, true); else NUPS_PUSH0(false, false, true); }
