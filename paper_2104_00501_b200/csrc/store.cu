@@ -367,17 +367,16 @@ struct TablePair {
     float4* out;           // [n][L]
 };
 
-template <bool HOT, bool TWO, bool F64>
+template <bool HOT, bool TWO, bool F64, bool PARTS>
 __global__ void __launch_bounds__(256, 4)
 gather_kernel(View v, const uint32_t* __restrict__ keys, uint64_t n, TablePair A, TablePair B, int map,
               uint64_t map_base, uint64_t map_total, int do_count, uint32_t* __restrict__ keys_copy, uint32_t parts)
 {
     grid_dependency_wait();
     const unsigned lane = threadIdx.x & 31;
-    const uint64_t team = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5, warp = team / parts;
-    const uint32_t part = (uint32_t)(team - warp * parts);         // this warp's share of the window's rows
-    const uint64_t nwarps = (((uint64_t)gridDim.x * blockDim.x) >> 5) / parts;
-    if (warp >= nwarps) return;
+    const uint64_t team = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5, teams = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+    const uint64_t warp = PARTS ? team / parts : team, nwarps = PARTS ? teams / parts : teams;
+    const uint32_t part = PARTS ? (uint32_t)(team - warp * parts) : 0u;            // this warp's share of the window's rows
     const uint32_t L4 = v.L4;
     // Lookups run ahead of the copies: while window w is copied, the key of window w + 2 and the
     // hot-bit word of window w + 1 are already on their way.
@@ -414,8 +413,8 @@ gather_kernel(View v, const uint32_t* __restrict__ keys, uint64_t n, TablePair A
                 if (cold_m) atomicAdd(&v.st->cold_hits, (unsigned long long)__popc(cold_m));
             }
         }
-        const int rows = (int)min((uint64_t)32, n - base), share = 32 / (int)parts;
-        for (int r = (int)part * share; r < min(rows, ((int)part + 1) * share); r += GATHER_UNROLL) {
+        const int rows = (int)min((uint64_t)32, n - base), share = PARTS ? 32 / (int)parts : 32;
+        for (int r = (int)part * share; r < (PARTS ? min(rows, ((int)part + 1) * share) : rows); r += GATHER_UNROLL) {
             unsigned long long so[GATHER_UNROLL], po[GATHER_UNROLL];
 #pragma unroll
             for (int u = 0; u < GATHER_UNROLL; ++u) {
@@ -461,7 +460,7 @@ gather_kernel(View v, const uint32_t* __restrict__ keys, uint64_t n, TablePair A
 // 32 / C8 whole rows, which halves the load/store instructions per byte.  Used when some keys are replicated: once
 // many rows come from L2 (hot or repeated keys) the copy is bound by the instructions its rows take in the
 // load/store pipe, not by DRAM.
-template <bool HOT, int C8>
+template <bool HOT, int C8, bool PARTS>
 __global__ void __launch_bounds__(256, 4)
 gather8_kernel(View v, const uint32_t* __restrict__ keys, uint64_t n, const float* __restrict__ table,
                const float* slab, float* __restrict__ out, int map, uint64_t map_base, uint64_t map_total, int do_count,
@@ -472,10 +471,9 @@ gather8_kernel(View v, const uint32_t* __restrict__ keys, uint64_t n, const floa
     constexpr int UNR = 2;                             // instructions in flight
     const unsigned lane = threadIdx.x & 31;
     const unsigned sub = lane / C8, c = lane % C8;     // which of the instruction's rows, which chunk of it
-    const uint64_t team = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5, warp = team / parts;
-    const uint32_t part = (uint32_t)(team - warp * parts);         // this warp's share of the window's rows
-    const uint64_t nwarps = (((uint64_t)gridDim.x * blockDim.x) >> 5) / parts;
-    if (warp >= nwarps) return;
+    const uint64_t team = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5, teams = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+    const uint64_t warp = PARTS ? team / parts : team, nwarps = PARTS ? teams / parts : teams;
+    const uint32_t part = PARTS ? (uint32_t)(team - warp * parts) : 0u;            // this warp's share of the window's rows
     const uint64_t L = (uint64_t)v.L4 * 4;
     const uint64_t stride = nwarps * 32;
     uint64_t base = warp * 32;
@@ -512,7 +510,7 @@ gather8_kernel(View v, const uint32_t* __restrict__ keys, uint64_t n, const floa
                 if (cold_m) atomicAdd(&v.st->cold_hits, (unsigned long long)__popc(cold_m));
             }
         }
-        const int share = 32 / (int)parts, rows = (int)min((uint64_t)((part + 1) * share), end - base);
+        const int share = PARTS ? 32 / (int)parts : 32, rows = (int)min((uint64_t)((part + 1) * share), end - base);
         for (int r0 = (int)part * share; r0 < rows; r0 += UNR * RPI) {
             uint32_t so[UNR], po[UNR];
             F8 a[UNR];
@@ -550,6 +548,7 @@ gather8_kernel(View v, const uint32_t* __restrict__ keys, uint64_t n, const floa
 // Into how many warps (a power of two, at most `most`) the rows of a window of 32 are divided, so that up to `resident` warps
 // have work.  A warp takes its rows a few at a time, one memory latency after the other, so the windows of a small call would
 // leave most multiprocessors idle while a few warps wait eight times in a row; every warp of a window repeats its lookups.
+// (The kernels of larger calls are built without the division, which took 0.5 % of a pull of 1M rows.)
 // Measured: pulling 50,000 rows of 100 floats 13.7 -> 9.9 us, pushing 5,000 10.3 -> 6.8 us, a round of pull and push over two
 // tables with 20,000 rows 43 -> 30 us.
 static uint32_t window_parts(uint64_t rows, uint64_t resident, uint32_t most)
@@ -584,7 +583,7 @@ nups_status nups_gather_internal(nups_store* s, const uint32_t* d_keys, uint64_t
         const float* slab = (const float*)A.slab;
         nups_time_begin(s, st, worker_map == 1 ? NUPS_TIMED_SAMPLE_ROWS : NUPS_TIMED_PULL);
 #define NUPS_G8(C8_)                                                                                                     \
-        nups_launch_dependent(gather8_kernel<true, C8_>, grid, 256, 0, st, v, d_keys, n, table, slab, out1, worker_map, map_base, map_total, \
+        nups_launch_dependent(parts > 1 ? gather8_kernel<true, C8_, true> : gather8_kernel<true, C8_, false>, grid, 256, 0, st, v, d_keys, n, table, slab, out1, worker_map, map_base, map_total, \
                                                         do_count, d_keys_copy, parts)
         if (c8 == 8) NUPS_G8(8);
         else if (c8 == 16) NUPS_G8(16);
@@ -596,7 +595,7 @@ nups_status nups_gather_internal(nups_store* s, const uint32_t* d_keys, uint64_t
     }
     nups_time_begin(s, st, worker_map == 1 ? NUPS_TIMED_SAMPLE_ROWS : NUPS_TIMED_PULL);
 #define NUPS_GATHER(HOT_, TWO_, F64_)                                                                                  \
-    nups_launch_dependent(gather_kernel<HOT_, TWO_, F64_>, grid, 256, 0, st, v, d_keys, n, A, B, worker_map, map_base, map_total, do_count, \
+    nups_launch_dependent(parts > 1 ? gather_kernel<HOT_, TWO_, F64_, true> : gather_kernel<HOT_, TWO_, F64_, false>, grid, 256, 0, st, v, d_keys, n, A, B, worker_map, map_base, map_total, do_count, \
                                                           d_keys_copy, parts)
     if (s->vb == 8) {                        // only replica reads add; rows without a replica are copied whatever they hold
         if (s->H) { if (two) NUPS_GATHER(true, true, true); else NUPS_GATHER(true, false, true); }
@@ -1470,33 +1469,43 @@ extern "C" nups_status nups_push(nups_store* s, const uint32_t* d_keys, uint64_t
 
 // ---------------------------------------------------------------------------------------------
 // sync: merge the workers' pending updates of every touched hot slot into the stored row,
-// worker 0 first, and clear them and the marks.  One warp per slot: its lanes read the workers' marks of
-// the slot with one load each, so only slots and replicas that were touched cost more than that.  (A thread per chunk that
-// reads every worker's mark, and a separate clearing of the marks, took 9.2 us for 1,000 slots and 8 workers; this 3.6 us.)
+// worker 0 first, and clear them and the marks.  A warp per slot reads the workers' marks with one load each,
+// so only slots and replicas that were touched cost more than that.  Rows wider than a warp are divided among
+// two to eight warps, but only as long as the multiprocessors can hold all of them at once.
+// Measured: 1,000 slots of 512 bytes and 8 workers 9.2 -> 3.6 us (before: a thread per chunk that read every mark, the marks
+// cleared by a launch of its own).  20,000 slots of 1,200 bytes: 33 us with a thread per chunk, again 33 us with four warps
+// per slot (four replica rows in flight each; 16 us more still with eight), 11 us with one.  3,000 slots of two tables of
+// 2,000 bytes: 160 us longer with one warp per slot than with two.
 // ---------------------------------------------------------------------------------------------
 template <bool F64>
 __global__ void __launch_bounds__(256)
-sync_kernel(View v, const uint32_t* __restrict__ hot_keys)
+sync_kernel(View v, const uint32_t* __restrict__ hot_keys, uint32_t per_slot)      // warps per slot: 1, 2, 4 or 8
 {
     grid_dependency_wait();
     constexpr unsigned FULL = 0xFFFFFFFFu;
     constexpr int U = 4;                                     // replica rows in flight
     const uint32_t lane = threadIdx.x & 31, L4 = v.L4;
-    const uint64_t slot = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (slot >= v.H) return;
-    const uint32_t key = __ldg(hot_keys + slot);
+    const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5, slot = warp / per_slot;
+    const uint32_t part = (uint32_t)(warp - slot * per_slot);
+    const bool real = slot < v.H;
+    const uint32_t key = real ? __ldg(hot_keys + slot) : 0u;
     uint32_t marks[8], touched = 0;                          // R <= 254: marks of workers 32 w ... 32 w + 31
 #pragma unroll
     for (int w = 0; w < 8; ++w) {
         marks[w] = 0u;
         if (32 * w >= v.R) continue;
         const uint32_t r = 32 * w + lane;
-        const bool set = r < v.R && v.dirty[(size_t)r * v.Hcap + slot] != 0u;
+        const bool set = real && r < v.R && v.dirty[(size_t)r * v.Hcap + slot] != 0u;
         marks[w] = __ballot_sync(FULL, set);
         touched += __popc(marks[w]);
-        if (set) v.dirty[(size_t)r * v.Hcap + slot] = 0u;
     }
+    if (per_slot > 1) __syncthreads();                       // a slot's warps, all of one block, have read its marks
     if (!touched) return;
+    if (part == 0) {
+#pragma unroll
+        for (int w = 0; w < 8; ++w)
+            if (marks[w] >> lane & 1u) v.dirty[(size_t)(32 * w + lane) * v.Hcap + slot] = 0u;
+    }
     const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
     const size_t worker_stride = (size_t)v.Hcap * L4;
 #pragma unroll
@@ -1504,7 +1513,7 @@ sync_kernel(View v, const uint32_t* __restrict__ hot_keys)
         float4* table = (float4*)(which ? v.acc : v.val);
         float4* slab = (float4*)(which ? v.dacc : v.dval);
         if (!table || !slab) continue;
-        for (uint32_t c = lane; c < L4; c += 32) {
+        for (uint32_t c = part * 32 + lane; c < L4; c += per_slot * 32) {
             float4* row = table + (uint64_t)key * L4 + c;
             const float4 old = *row;
             float4 sum = zero;
@@ -1544,8 +1553,10 @@ nups_status nups_sync_internal(nups_store* s, cudaStream_t st)
     if (s->H == 0) return NUPS_OK;        // nothing replicated: no work at all
     View v = nups_view(s);
     nups_background_begin(s, st);
-    if (s->vb == 8) nups_launch_dependent(sync_kernel<true>, grid_for(s->H, 8), 256, 0, st, v, s->hot_keys);
-    else nups_launch_dependent(sync_kernel<false>, grid_for(s->H, 8), 256, 0, st, v, s->hot_keys);
+    uint32_t per_slot = 1;
+    while (per_slot < 8 && per_slot * 32 < v.L4 && s->H * per_slot * 2 <= (uint64_t)s->sm_count * 64) per_slot *= 2;
+    if (s->vb == 8) nups_launch_dependent(sync_kernel<true>, grid_for(s->H * per_slot, 8), 256, 0, st, v, s->hot_keys, per_slot);
+    else nups_launch_dependent(sync_kernel<false>, grid_for(s->H * per_slot, 8), 256, 0, st, v, s->hot_keys, per_slot);
     const cudaError_t e = cudaGetLastError();
     nups_background_end(s, st);
     if (e != cudaSuccess) return nups_cuda_fail(e, "replica merge");
