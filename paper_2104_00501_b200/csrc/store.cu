@@ -2152,6 +2152,14 @@ static nups_status grow_hot(nups_store* s, uint64_t need)
     return NUPS_OK;
 }
 
+// The stream is waited for once, at the latest when the call returns, whatever way it returns: the caller may hand the key list
+// on, or look at the store from another stream.
+static nups_status return_waited(cudaStream_t st, nups_status rc)
+{
+    CK(cudaStreamSynchronize(st));
+    return rc;
+}
+
 extern "C" nups_status nups_set_management(nups_store* s, const uint32_t* d_keys, uint64_t n, int technique, void* stream)
 {
     if (!s || (n && !d_keys) || (technique != NUPS_SINGLE && technique != NUPS_REPLICATE)) return NUPS_EINVAL;
@@ -2159,10 +2167,7 @@ extern "C" nups_status nups_set_management(nups_store* s, const uint32_t* d_keys
     cudaStream_t st = (cudaStream_t)stream;
     nups_status rc = nups_sync_internal(s, st);
     if (rc != NUPS_OK) return rc;
-    if (n == 0) {
-        CK(cudaStreamSynchronize(st));
-        return NUPS_OK;
-    }
+    if (n == 0) return return_waited(st, NUPS_OK);
     // no background merge may be enqueued or running while slots and replicas are rebuilt
     struct Bracket {
         nups_store* s;
@@ -2174,14 +2179,14 @@ extern "C" nups_status nups_set_management(nups_store* s, const uint32_t* d_keys
     size_t need = 2 * align256(m * 8) + align256(m * 4) + nups_scan_scratch_bytes(m) + 256;
     char* sc;
     rc = nups_scratch(s, need, &sc);
-    if (rc != NUPS_OK) return rc;
+    if (rc != NUPS_OK) return return_waited(st, rc);
     unsigned long long* flag = (unsigned long long*)sc; sc += align256(m * 8);
     unsigned long long* pos = (unsigned long long*)sc; sc += align256(m * 8);
     uint32_t* hk_new = (uint32_t*)sc; sc += align256(m * 4);
     unsigned long long* d_total = (unsigned long long*)sc; sc += 256;
     unsigned long long total = 0;
     if (technique == NUPS_REPLICATE) {
-        if (s->H + n >= (1ull << 31)) return NUPS_ENOMEM;
+        if (s->H + n >= (1ull << 31)) return return_waited(st, NUPS_ENOMEM);
         if (s->H + n > s->Hcap) CK(cudaStreamSynchronize(st));           // the merge is done before the replicas move
         rc = grow_hot(s, s->H + n);
         if (rc != NUPS_OK) return rc;
@@ -2208,7 +2213,7 @@ extern "C" nups_status nups_set_management(nups_store* s, const uint32_t* d_keys
     } else {
         demote_kernel<<<grid_for(n, 256), 256, 0, st>>>(s->slot_of, s->hot_bits, s->num_keys, d_keys, n, s->st);
         LAUNCH_CHECK(s);
-        if (s->H == 0) return NUPS_OK;
+        if (s->H == 0) return return_waited(st, NUPS_OK);
         if (s->H <= SMALL_LIST_KEYS) {
             renumber_small_kernel<<<1, MANAGE_THREADS, 0, st>>>(s->slot_of, s->hot_keys, (unsigned)s->H, d_total);
             LAUNCH_CHECK(s);

@@ -78,3 +78,33 @@ def test_lists_around_the_one_block_limit(n):
             s.set_management(dev_keys(keys), technique[1])
             assert np.array_equal(host_keys(s.hot_keys()), o.hot_keys())
     s.close()
+
+
+def test_setting_the_management_leaves_the_stream_idle():
+    # whatever way the call returns: nothing replicated, an empty list, a refused list, the ordinary ways
+    nk = 100_000
+    s = binding.Store(nk, 8, workers=4, max_device_mib=12)
+    few, many = dev_keys(np.arange(64)), dev_keys(np.arange(80_000))
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+
+    def idle_after(keys, technique, refused=False):
+        with torch.cuda.stream(stream):
+            torch.cuda._sleep(100_000_000)                          # about 50 ms that the call has to wait for
+            if refused:
+                with pytest.raises(binding.NupsError) as e:
+                    s.set_management(keys, technique)
+                assert e.value.code == binding.ENOMEM
+            else:
+                s.set_management(keys, technique)
+            return stream.query()
+
+    assert idle_after(few, binding.SINGLE)                          # no key is replicated
+    assert idle_after(few[:0], binding.REPLICATE)
+    assert idle_after(many, binding.REPLICATE, refused=True)        # 13 MB of replicas
+    assert idle_after(few, binding.REPLICATE)
+    assert idle_after(many, binding.REPLICATE, refused=True)
+    assert idle_after(few[:10].contiguous(), binding.SINGLE)
+    assert s.stats()["hot_slots"] == 54
+    stream.synchronize()
+    s.close()
