@@ -179,6 +179,8 @@ __device__ __forceinline__ void grid_dependency_wait()
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;");
 }
+// The wait alone: the next kernel becomes resident when this one's blocks are done.
+__device__ __forceinline__ void grid_dependency_wait_alone() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 template <class... KArgs, class... Args>
 static inline cudaError_t nups_launch_dependent(void (*kernel)(KArgs...), dim3 grid, unsigned block, size_t smem,
@@ -222,7 +224,8 @@ nups_status nups_gather_internal(nups_store* s, const uint32_t* d_keys, uint64_t
                                  float* d_out_acc, int worker_map, uint64_t map_base, uint64_t map_total,
                                  int do_count, cudaStream_t st,
                                  uint32_t* d_keys_copy /* nullable: also write the keys here */);
-nups_status nups_sync_internal(nups_store* s, cudaStream_t st);
+// early_next: the kernel that follows on the stream may become resident while the merge runs (see sync_kernel)
+nups_status nups_sync_internal(nups_store* s, cudaStream_t st, bool early_next = false);
 // sampling.cu internals used by steps.cu
 nups_status nups_draw_negatives(nups_store* s, int32_t dist, uint64_t N, cudaStream_t st);
 nups_status nups_sample_ahead_rewind(nups_store* s, cudaStream_t st);

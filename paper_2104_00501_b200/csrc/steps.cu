@@ -1339,12 +1339,12 @@ extern "C" nups_status nups_run_sgns(nups_store* s, const uint32_t* d_center, co
             if (t < steps) {
                 CK(cudaEventRecord(s->side_fork, st));
                 CK(cudaStreamWaitEvent(s->side, s->side_fork, 0));
-                rc = nups_sync_internal(s, s->side);
+                rc = nups_sync_internal(s, s->side, true);
                 if (rc != NUPS_OK) return rc;
                 CK(cudaEventRecord(s->side_join, s->side));
                 merge_in_flight = true;
             } else {
-                rc = nups_sync_internal(s, st);
+                rc = nups_sync_internal(s, st, true);                     // next comes, as a rule, the next call's draw
                 if (rc != NUPS_OK) return rc;
             }
         }

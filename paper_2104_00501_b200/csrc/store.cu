@@ -1476,12 +1476,18 @@ extern "C" nups_status nups_push(nups_store* s, const uint32_t* d_keys, uint64_t
 // cleared by a launch of its own).  20,000 slots of 1,200 bytes: 33 us with a thread per chunk, again 33 us with four warps
 // per slot (four replica rows in flight each; 16 us more still with eight), 11 us with one.  3,000 slots of two tables of
 // 2,000 bytes: 160 us longer with one warp per slot than with two.
+// The next kernel of the stream waits for the merge's end before its blocks become resident, unless the caller knows that
+// it is a small one: a push or a step whose blocks fill the multiprocessors runs longer when they were placed between the
+// merge's.  Measured, placed between them and after them: 1M rows pushed and 1,000 slots merged, in turn, 200 and 191 us;
+// ComplEx steps of three stores in turn, every 16th with a merge, 229 and 225 us each.  Skip-gram steps, whose merges are
+// followed by a draw or by an event: 456.7 and 457.7 us for 64 of them.
 // ---------------------------------------------------------------------------------------------
 template <bool F64>
 __global__ void __launch_bounds__(256)
-sync_kernel(View v, const uint32_t* __restrict__ hot_keys, uint32_t per_slot)      // warps per slot: 1, 2, 4 or 8
+sync_kernel(View v, const uint32_t* __restrict__ hot_keys, uint32_t per_slot, bool early_next)      // warps per slot: 1, 2, 4 or 8
 {
-    grid_dependency_wait();
+    if (early_next) grid_dependency_wait();
+    else grid_dependency_wait_alone();
     constexpr unsigned FULL = 0xFFFFFFFFu;
     constexpr int U = 4;                                     // replica rows in flight
     const uint32_t lane = threadIdx.x & 31, L4 = v.L4;
@@ -1548,15 +1554,15 @@ sync_kernel(View v, const uint32_t* __restrict__ hot_keys, uint32_t per_slot)   
     }
 }
 
-nups_status nups_sync_internal(nups_store* s, cudaStream_t st)
+nups_status nups_sync_internal(nups_store* s, cudaStream_t st, bool early_next)
 {
     if (s->H == 0) return NUPS_OK;        // nothing replicated: no work at all
     View v = nups_view(s);
     nups_background_begin(s, st);
     uint32_t per_slot = 1;
     while (per_slot < 8 && per_slot * 32 < v.L4 && s->H * per_slot * 2 <= (uint64_t)s->sm_count * 64) per_slot *= 2;
-    if (s->vb == 8) nups_launch_dependent(sync_kernel<true>, grid_for(s->H * per_slot, 8), 256, 0, st, v, s->hot_keys, per_slot);
-    else nups_launch_dependent(sync_kernel<false>, grid_for(s->H * per_slot, 8), 256, 0, st, v, s->hot_keys, per_slot);
+    if (s->vb == 8) nups_launch_dependent(sync_kernel<true>, grid_for(s->H * per_slot, 8), 256, 0, st, v, s->hot_keys, per_slot, early_next);
+    else nups_launch_dependent(sync_kernel<false>, grid_for(s->H * per_slot, 8), 256, 0, st, v, s->hot_keys, per_slot, early_next);
     const cudaError_t e = cudaGetLastError();
     nups_background_end(s, st);
     if (e != cudaSuccess) return nups_cuda_fail(e, "replica merge");
