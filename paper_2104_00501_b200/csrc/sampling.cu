@@ -636,14 +636,15 @@ __device__ __forceinline__ LtChunk lt_chunk(uint32_t q, uint64_t N, uint32_t R, 
     return c;
 }
 
-// Lookups and scan in one launch, as the calls are bound by their launches: 120,000 samples pulled in four parts 86 -> 73 us
-// with this and the rows copied by the placement pass; 1M samples in one part 124 -> 130 us (the fences).  A block that has
-// written its bits makes them visible and takes a ticket; the one that draws the last of its sub-handle's tickets sees all
-// of them and scans.  Nobody waits for anybody.
+// Lookups and scan in one launch, as the calls are bound by their launches: drawing 120,000 samples and pulling them in four
+// parts 91 -> 74 us with this and the rows copied by the placement pass, 1M samples in one part 134 -> 130 us, in four 186 -> 184 us
+// (135 and 193 us with twice as many blocks as are resident).  A block that has written its bits makes them visible and takes
+// a ticket; the one that draws the last of its sub-handle's tickets sees all of them and scans.  Nobody waits for anybody.
 constexpr int LT_THREADS = 512;
+constexpr unsigned LT_BLOCKS = 2;            // resident per multiprocessor
 constexpr int LT_WORDS = 4;                  // flag words per thread and round of the scan
 
-__global__ void __launch_bounds__(LT_THREADS)
+__global__ void __launch_bounds__(LT_THREADS, LT_BLOCKS)
 lt_walk_kernel(View v, HandleView h, uint64_t N, uint64_t cursor, uint64_t n, uint32_t q_first)
 {
     grid_dependency_wait();
@@ -850,7 +851,8 @@ static nups_status pull_internal(nups_store* s, int id, uint64_t n, uint32_t* d_
         // words of a sub-handle and of its postponed entries: together at most three more than the sub-handle's entries fill
         const dim3 by_word(grid_for(max_size / 32 + 4, 8), ql - qf + 1);
         // as many blocks as are resident at once: every block pays for a fence and a ticket
-        const unsigned walkers = grid_for(max_size / 32 + 2, LT_THREADS / 32, grid_for((uint64_t)s->sm_count * 4, ql - qf + 1));
+        const unsigned resident = (unsigned)s->sm_count * LT_BLOCKS / (ql - qf + 1);
+        const unsigned walkers = grid_for(max_size / 32 + 2, LT_THREADS / 32, resident ? resident : 1);
         nups_launch_dependent(lt_walk_kernel, dim3(walkers, ql - qf + 1), LT_THREADS, 0, st, v, hv, h.N, h.cursor, n, qf);
         LAUNCH_CHECK(s);
         // the placement pass can copy the rows itself (one table of 64, 128 or 256 floats per row, 32-byte aligned output)
