@@ -1471,20 +1471,21 @@ extern "C" nups_status nups_push(nups_store* s, const uint32_t* d_keys, uint64_t
 // sync: merge the workers' pending updates of every touched hot slot into the stored row,
 // worker 0 first, and clear them and the marks.  A warp per slot reads the workers' marks with one load each,
 // so only slots and replicas that were touched cost more than that.  Rows wider than a warp are divided among
-// two to eight warps, but only as long as the multiprocessors hold all of them at once (SYNC_BLOCKS blocks each).
+// two to eight warps as long as they make at most two waves (of 32 warps per multiprocessor: the kernel takes 56 to 60 registers).
 // Measured: 1,000 slots of 512 bytes and 8 workers 9.2 -> 3.6 us (before: a thread per chunk that read every mark, the marks
 // cleared by a launch of its own).  All replicas of two tables of 2,000 bytes touched, launch and events included, with 1, 2
 // and 4 warps per slot: 300 slots 17.6, 12.5, 10.9 us; 1,200 slots 21.4, 16.9, 18.6; 2,400 slots 31.6, 33.7, 29.2; 4,000 bytes,
-// one table, 300 slots with 1 and 8: 17.5, 10.2.  20,000 slots of 1,200 bytes with 1 and 4: 11 and 33 us.
+// one table, 300 slots with 1 and 8: 17.5, 10.2.  20,000 slots of 1,200 bytes with 1 and 4: 11 and 33 us.  The second wave pays
+// among other work: 50,000 rows of two such tables pulled, pushed and merged, 1,200 slots: 219.7 us, with one wave 222.9;
+// 2,400 slots: 228.6 and 235.0.  (Held to 64 registers the kernel merges 1,000 slots of 1,024 bytes 8 us slower.)
 // The next kernel of the stream waits for the merge's end before its blocks become resident, unless the caller knows that
 // it is a small one: a push or a step whose blocks fill the multiprocessors runs longer when they were placed between the
 // merge's.  Measured, placed between them and after them: 1M rows pushed and 1,000 slots merged, in turn, 200 and 191 us;
 // ComplEx steps of three stores in turn, every 16th with a merge, 229 and 225 us each.  Skip-gram steps, whose merges are
 // followed by a draw or by an event: 456.7 and 457.7 us for 64 of them.
 // ---------------------------------------------------------------------------------------------
-constexpr unsigned SYNC_BLOCKS = 4;          // of 256 threads, resident per multiprocessor
 template <bool F64>
-__global__ void __launch_bounds__(256, SYNC_BLOCKS)
+__global__ void __launch_bounds__(256)
 sync_kernel(View v, const uint32_t* __restrict__ hot_keys, uint32_t per_slot, bool early_next)      // warps per slot: 1, 2, 4 or 8
 {
     if (early_next) grid_dependency_wait();
@@ -1561,7 +1562,7 @@ nups_status nups_sync_internal(nups_store* s, cudaStream_t st, bool early_next)
     View v = nups_view(s);
     nups_background_begin(s, st);
     uint32_t per_slot = 1;
-    while (per_slot < 8 && per_slot * 32 < v.L4 && s->H * per_slot * 2 <= (uint64_t)s->sm_count * SYNC_BLOCKS * 8) per_slot *= 2;
+    while (per_slot < 8 && per_slot * 32 < v.L4 && s->H * per_slot * 2 <= (uint64_t)s->sm_count * 64) per_slot *= 2;
     if (s->vb == 8) nups_launch_dependent(sync_kernel<true>, grid_for(s->H * per_slot, 8), 256, 0, st, v, s->hot_keys, per_slot, early_next);
     else nups_launch_dependent(sync_kernel<false>, grid_for(s->H * per_slot, 8), 256, 0, st, v, s->hot_keys, per_slot, early_next);
     const cudaError_t e = cudaGetLastError();

@@ -12,8 +12,8 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("L,value_bytes,two,R,hot_n", [
-    (1028, 4, False, 40, 60), (1028, 4, True, 3, 592), (1028, 4, False, 3, 593), (600, 8, True, 40, 50), (500, 4, True, 5, 1184),
-    (500, 4, True, 5, 1185), (260, 4, False, 2, 2368), (260, 4, False, 2, 2369), (128, 4, True, 254, 20), (132, 8, False, 33, 30)])
+    (1028, 4, False, 40, 60), (1028, 4, True, 3, 1184), (1028, 4, False, 3, 1185), (600, 8, True, 40, 50), (500, 4, True, 5, 2368),
+    (500, 4, True, 5, 2369), (260, 4, False, 2, 2368), (260, 4, False, 2, 2369), (128, 4, True, 254, 20), (132, 8, False, 33, 30)])
 def test_the_merged_tables_are_the_oracles(L, value_bytes, two, R, hot_n):
     nk = 4000
     rng = np.random.default_rng(L + R)
