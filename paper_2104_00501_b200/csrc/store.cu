@@ -1633,6 +1633,18 @@ extern "C" nups_status nups_count_accesses(nups_store* s, const uint32_t* d_keys
     return NUPS_OK;
 }
 
+// Is p memory of the store's GPU, which a kernel may write to?  Results go anywhere else (another GPU, the host) by the copy
+// call, which finds its way there or returns an error.
+static bool own_memory(const nups_store* s, const void* p)
+{
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return at.type == cudaMemoryTypeDevice && at.device == s->device;
+}
+
 // The counts are handed out by a copy of our own: they are next to the multiprocessors in L2 when they have just been
 // counted or chosen from, and reading 64 bytes per thread at once takes them out faster than the copy call (88 MB: 42 us, 50 us).
 __global__ void __launch_bounds__(256)
@@ -1652,7 +1664,7 @@ extern "C" nups_status nups_get_counts(nups_store* s, uint64_t* d_out, void* str
 {
     if (!s || !d_out) return NUPS_EINVAL;
     cudaStream_t st = (cudaStream_t)stream;
-    if ((uintptr_t)d_out & 15) {                             // not aligned for wide stores
+    if (!own_memory(s, d_out) || ((uintptr_t)d_out & 15)) {  // ... or not aligned for wide stores
         CK(cudaMemcpyAsync(d_out, s->cnt, s->num_keys * 8, cudaMemcpyDeviceToDevice, st));
         return NUPS_OK;
     }
@@ -1961,8 +1973,10 @@ extern "C" nups_status nups_select_hot(nups_store* s, int by_topk, uint64_t para
     uint32_t* order;
     rc = sort_passes<unsigned long long>(s, k0, v0, k1, v1, hist, plan, st, &sorted, &order);
     if (rc != NUPS_OK) return rc;
-    nups_launch_dependent(select_out_kernel, grid_for(take, 256), 256, 0, st, keys, order, take, d_keys_out);
+    uint32_t* out = own_memory(s, d_keys_out) ? d_keys_out : order == v0 ? v1 : v0;
+    nups_launch_dependent(select_out_kernel, grid_for(take, 256), 256, 0, st, keys, order, take, out);
     LAUNCH_CHECK(s);
+    if (out != d_keys_out) CK(cudaMemcpyAsync(d_keys_out, out, take * 4, cudaMemcpyDeviceToDevice, st));
     CK(cudaStreamSynchronize(st));
     *h_n_out = take;
     return NUPS_OK;

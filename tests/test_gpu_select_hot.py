@@ -1,5 +1,7 @@
 """Counting, choosing and managing hot keys at the sizes where the parts hand over: the block's own table of keys, bins of
 counts that are cut finer, ties on the lowest chosen count, stretches of keys, and lists around the one-block limit."""
+import ctypes as C
+
 import numpy as np
 import pytest
 import torch
@@ -107,4 +109,32 @@ def test_setting_the_management_leaves_the_stream_idle():
     assert idle_after(few[:10].contiguous(), binding.SINGLE)
     assert s.stats()["hot_slots"] == 54
     stream.synchronize()
+    s.close()
+
+
+def test_results_are_copied_where_no_kernel_should_write():
+    # page-locked host memory stands for all memory that is not the store's GPU's: no kernel writes the counts to it
+    nk = 5001
+    rng = np.random.default_rng(1)
+    s = binding.Store(nk, 4, sync_interval=0)
+    keys = (rng.zipf(1.3, 20_000) % nk).astype(np.uint32)
+    s.count_accesses(dev_keys(keys))
+    counts = np.bincount(keys, minlength=nk)
+    lib, h, stream = binding.load(), s._s, torch.cuda.current_stream()
+    out = torch.zeros(nk, dtype=torch.int64).pin_memory()
+    before = s.stats()["launches"]
+    assert lib.nups_get_counts(h, out.data_ptr(), stream.cuda_stream) == binding.OK
+    assert s.stats()["launches"] == before
+    stream.synchronize()
+    assert np.array_equal(out.numpy(), counts)
+    for off in (0, 1):                                               # the GPU's own memory, also where 16-byte stores do not fit
+        buf = torch.zeros(nk + 1, dtype=torch.int64, device="cuda")
+        assert lib.nups_get_counts(h, buf[off:].data_ptr(), stream.cuda_stream) == binding.OK
+        assert np.array_equal(buf[off:off + nk].cpu().numpy(), counts)
+    hot, n = torch.zeros(nk, dtype=torch.int32).pin_memory(), C.c_uint64()
+    for by_topk, param, want in ((1, 100, 100), (0, 1, int((counts * nk > counts.sum()).sum()))):
+        assert lib.nups_select_hot(h, by_topk, param, hot.data_ptr(), C.byref(n), stream.cuda_stream) == binding.OK
+        assert n.value == want
+        assert np.array_equal(hot.numpy()[:want].view(np.uint32), _top(counts, want))
+    assert s.status_check() == 0
     s.close()
