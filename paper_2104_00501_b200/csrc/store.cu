@@ -1117,6 +1117,9 @@ push_apply_kernel(View v, const K* __restrict__ dest, const uint32_t* __restrict
 constexpr unsigned CHAIN_THREADS = 160, CHAIN_STAGES = 6, CHAIN_STAGE_BYTES = 8192;
 constexpr unsigned CHAIN_SMEM = CHAIN_STAGES * CHAIN_STAGE_BYTES;  // 48 KB: four blocks per multiprocessor
 
+// The copying warps and the adding warp meet here, at different places of the kernel, once per stage.
+__device__ __forceinline__ void chain_stage_barrier() { asm volatile("bar.sync 1, %0;" ::"n"(CHAIN_THREADS) : "memory"); }
+
 template <class K, bool F64>
 __global__ void __launch_bounds__(CHAIN_THREADS)
 push_chain_kernel(View v, const K* __restrict__ dest, const uint32_t* __restrict__ idx, uint64_t n,
@@ -1174,7 +1177,7 @@ push_chain_kernel(View v, const K* __restrict__ dest, const uint32_t* __restrict
                     const uint32_t stage = stage0 + l;
                     if (stage >= CHAIN_STAGES - 1 && stage < stages + CHAIN_STAGES - 1) {
                         asm volatile("cp.async.wait_group %0;" ::"n"(CHAIN_STAGES - 2) : "memory");
-                        __syncthreads();                           // stage - (CHAIN_STAGES - 1) is there, the one before it added up
+                        chain_stage_barrier();                     // stage - (CHAIN_STAGES - 1) is there, the one before it added up
                     }
                     const uint32_t to = ring_s + stage % CHAIN_STAGES * CHAIN_STAGE_BYTES + t * 16;
 #pragma unroll
@@ -1190,7 +1193,7 @@ push_chain_kernel(View v, const K* __restrict__ dest, const uint32_t* __restrict
         }
         if (adds)
         for (uint32_t stage = 0; stage < stages; ++stage) {
-            __syncthreads();
+            chain_stage_barrier();
             const V* x = reinterpret_cast<const V*>(ring + stage % CHAIN_STAGES * CHAIN_STAGE_BYTES) + lane;
             const uint32_t left = min(rows - stage * ROWS, ROWS);
             uint32_t r = 0;
