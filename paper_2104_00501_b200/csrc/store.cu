@@ -71,7 +71,9 @@ void nups_dev_free(nups_store* s, void* p, size_t bytes)
 nups_status nups_scratch(nups_store* s, size_t bytes, char** out)
 {
     if (bytes > s->scratch_bytes) {
-        size_t want = bytes + bytes / 4 + (1u << 20);
+        // some to spare: a quarter and 1,000 KiB.  (The rest of a MiB is left for the fixed parts of a choice of hot keys, which
+        // at a few keys take up to 15 KB more than sorting all keys does, so that a limit does not refuse it for them.)
+        size_t want = bytes + bytes / 4 + (1000u << 10);
         // the limit is judged with the old buffer already handed back; on refusal the old buffer stays
         if (s->dev_cap && (want > s->dev_cap || s->dev_bytes - s->scratch_bytes > s->dev_cap - want)) return NUPS_ENOMEM;
         nups_dev_free(s, s->scratch, s->scratch_bytes);
@@ -1323,7 +1325,7 @@ static unsigned long long invalid_dest(const nups_store* s) { return s->num_keys
 
 size_t nups_push_scratch_bytes(const nups_store* s, uint64_t n)
 {
-    if (!s->cfg.deterministic) return 0;
+    if (!s->cfg.deterministic || (narrow_dest(s) && n <= SMALL_PUSH_ROWS)) return 0;     // push_small_kernel needs none
     const size_t key = narrow_dest(s) ? 4 : 8;
     return 2 * align256(n * key) + 2 * align256(n * 4) + align256((sort_plan(n, bits_for(invalid_dest(s))).hist_words() + 1) * 4);
 }

@@ -61,6 +61,19 @@ def test_every_allocating_call_respects_the_stores_limit_and_leaves_the_store_us
     s.close()
 
 
+def test_small_calls_fit_under_a_limit_that_leaves_little_more_than_a_mebibyte():
+    # one row of 192,684 floats and the store's fixed 0.26 MB leave 1.06 MB of the 2 MiB: what sorting a few keys or rows
+    # takes with a MiB to spare
+    L = 192_684
+    s = binding.Store(1, L, workers=1, deterministic=True, max_device_mib=2)
+    s.count_accesses(dev_keys(np.zeros(5, np.uint32)))
+    assert host_keys(s.select_hot(True, 1)).tolist() == [0]
+    assert host_keys(s.select_hot(False, 0)).tolist() == [0]
+    s.push(dev_keys(np.zeros(3, np.uint32)), torch.ones((3, L), device="cuda"))
+    assert bool((s.read_table() == 3).all())
+    s.close()
+
+
 @pytest.mark.parametrize("level", [BOUNDED, LONGTERM])
 def test_ownership_survives_the_wrap_of_the_call_counter(level):
     # calls that move keys are numbered with 24 bits inside the ownership words; start three calls before the
