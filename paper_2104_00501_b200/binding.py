@@ -137,7 +137,8 @@ def _ptr(t, dtype=None):
 
 def _stream():
     # the current device's current stream as a number, without the Stream object that torch.cuda.current_stream() makes
-    # (1.5 us of the 5 us that a small call spends in Python); a Store has initialised CUDA by then
+    # (a pull of 96 rows spends 10.6 us on the host with the object, 3.3 of them on it, and 6.8 us this way); a Store has
+    # initialised CUDA by then
     return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 

@@ -368,7 +368,8 @@ __global__ void draw_iid_kernel(View v, DrawParams p, const unsigned long long* 
 // before it, which is what position j held before step j if j > i was the last step to write there (r_j = r_i), and r_i
 // itself if none was; and likewise for position j.  So the warp takes 32 steps at once and notes for each the last step
 // before it that wrote position r_i: one of the 32, found by comparing the r_i bit by bit with ballots, or what the steps
-// before left in last[r_i].  All positions then follow these notes side by side (at most 5 of them for 250 positions).
+// before left in last[r_i].  All positions then follow these notes side by side.  (The longest chain of notes of a shuffle
+// has no bound below G; over 2,000 shuffles of 250 positions it was 6.6 on average and 14 at most, of 1,024 positions 8.7 and 15.)
 // Measured, pools of 250 with 16 passes: 19 -> 14 us for 1M samples, 16 -> 10 us for sixteen batches of 12,288, where one thread
 // per pass made the swaps (11,000 of 22,000 cycles; noting the steps one by one still takes 8,500).
 // Shared memory: pool[G] (u32) | step[T][P] (u16) | last[T][P] (u16).

@@ -1904,7 +1904,7 @@ extern "C" nups_status nups_select_hot(nups_store* s, int by_topk, uint64_t para
     CK(cudaMemcpyAsync(&stat, d_stat, sizeof(stat), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
     const unsigned long long total = stat.sum, max_cnt = stat.max;
-    if (bits_for(n - 1) + bits_for(max_cnt) > 64) return NUPS_ESTATE;
+    if (bits_for(n - 1) + bits_for(max_cnt) > 64) return NUPS_ESTATE;        // the call's documented limit, not this method's
     // keys above `cut` are chosen, and the first `ties` of those on it; m = how many that makes, `take` of them are wanted
     unsigned long long cut = 0, ties = 0;
     uint64_t m = 0, take = 0;

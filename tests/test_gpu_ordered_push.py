@@ -1,5 +1,5 @@
 """The ordered push at the sizes where its parts hand over to one another: the launch without a sort up to 3,072 rows, tiles
-and rounds of the sort, windows of 32 sorted rows, destinations with more than 32 rows, and their ring of 12 stages."""
+and rounds of the sort, windows of 8, 16 or 32 sorted rows, destinations with more than 32 rows, and their ring of 6 stages."""
 import numpy as np
 import pytest
 import torch

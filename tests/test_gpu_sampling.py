@@ -142,11 +142,11 @@ def test_large_handles_with_most_keys_taken_by_other_workers(level):
     assert s.status_check() == 0
 
 
-@pytest.mark.parametrize("L", [64, 128, 256])
+@pytest.mark.parametrize("L", [64, 128, 256, 100])
 def test_full_pull_with_values_under_postponing_copies_the_rows_itself(L):
-    # rows of 64 / 128 / 256 floats: a full PullSample of a fresh LONG-TERM handle places keys and copies rows in one
-    # pass; replicated keys carry unmerged updates, ownership has been stirred, and a second handle is pulled in parts
-    # (the separate gather) for comparison with the same oracle
+    # rows of 64 / 128 / 256 floats: a PullSample of a LONG-TERM handle places keys and copies rows in one pass, whole or
+    # in parts; rows of 100 floats are copied by the separate gather.  Replicated keys carry unmerged updates, ownership
+    # has been stirred, and a second handle is pulled in parts
     nk, R, N = 5000, 4, 20_000
     rng = np.random.default_rng(L)
     init = rng.normal(size=(nk, L)).astype(np.float32)
