@@ -65,10 +65,10 @@ NCU_TRAFFIC = {"bytes_per_launch": 38886656 + 4509952, "sgns_kernel_sha1": "a667
 # kernel's source text at the time.  The traffic reported for the timed launch is scaled by the algorithmic bytes, which is
 # what the capture shows the traffic follows.  A kernel whose source has changed since reports no traffic.
 NCU_TRAFFIC_PS = {
-    "pull": {"dram_bytes": 216757504 + 481016320, "algorithmic_bytes": 694418688, "sha1": "d6be6ab4363bba8db6eba30551f6fe4750727ba0"},
-    "push": {"dram_bytes": 712619776 + 126636032, "algorithmic_bytes": 847772160, "sha1": "0a8c080becb64f3aaf867fbcd3f9c9bc21bc1399"},
-    "sample_rows": {"dram_bytes": 27681024 + 478645504, "algorithmic_bytes": 562094080,
-                    "sha1": "d6be6ab4363bba8db6eba30551f6fe4750727ba0"},
+    "pull": {"dram_bytes": 216990208 + 481212928, "algorithmic_bytes": 694418688, "sha1": "deb2f8ae2e333874a327aaa289dae4675801e5c8"},
+    "push": {"dram_bytes": 712659712 + 126633728, "algorithmic_bytes": 847772160, "sha1": "e181b4084e7f48a8f1df95f473809540f38216e4"},
+    "sample_rows": {"dram_bytes": 27697152 + 478537216, "algorithmic_bytes": 562094080,
+                    "sha1": "deb2f8ae2e333874a327aaa289dae4675801e5c8"},
 }
 PS_KERNEL_SOURCE = {   # kind -> (kernel name, start and end markers of its source text in store.cu)
     "pull": ("gather8_kernel", "// The same gather with 256-bit loads and stores", "nups_status nups_gather_internal("),
@@ -1110,7 +1110,9 @@ def run_step_workload(args, device, which, emit=True):
     # at the copy peak) and every update is a floating-point reduction to a DRAM-resident row, whose rate the library
     # measures by itself.  floor = both in full overlap, read_then_reduce = one after the other.
     red_dram = s.probe_reduction_rate(2 << 30, 5)
-    t_read, t_red = (logical / 2) / (hbm_peak * 1e9), (logical / 2) / (red_dram * 1e9)
+    # (Cells in column order: the column's row stays in registers, so a cell reads and updates one row.)
+    moved = logical / 2 / (2 if which == "mf" and args.mf_order == "column" else 1)
+    t_read, t_red = moved / (hbm_peak * 1e9), moved / (red_dram * 1e9)
     line = {"workload": cfg, "kernel": name, "hot_slots": s.stats()["hot_slots"], "us_per_step": dt * 1e6,
             "kernel_us": k_s * 1e6, "key_accesses_per_s": B * per_item / dt, "updates_per_s": B * upd / dt,
             "logical_gbs": logical / k_s / 1e9, "logical_frac_of_hbm_peak": logical / k_s / 1e9 / hbm_peak,
