@@ -71,11 +71,13 @@ void nups_dev_free(nups_store* s, void* p, size_t bytes)
 nups_status nups_scratch(nups_store* s, size_t bytes, char** out)
 {
     if (bytes > s->scratch_bytes) {
-        // some to spare: a quarter and 1,000 KiB.  (The rest of a MiB is left for the fixed parts of a choice of hot keys, which
-        // at a few keys take up to 15 KB more than sorting all keys does, so that a limit does not refuse it for them.)
-        size_t want = bytes + bytes / 4 + (1000u << 10);
+        size_t want = bytes + bytes / 4 + (1u << 20);
         // the limit is judged with the old buffer already handed back; on refusal the old buffer stays
-        if (s->dev_cap && (want > s->dev_cap || s->dev_bytes - s->scratch_bytes > s->dev_cap - want)) return NUPS_ENOMEM;
+        auto refused = [&]() { return s->dev_cap && (want > s->dev_cap || s->dev_bytes - s->scratch_bytes > s->dev_cap - want); };
+        // less to spare under a tight limit: the fixed parts of a choice among few hot keys take up to 15 KB more than sorting
+        // all keys does, and are not to be what the limit refuses
+        if (refused()) want -= 24u << 10;
+        if (refused()) return NUPS_ENOMEM;
         nups_dev_free(s, s->scratch, s->scratch_bytes);
         s->scratch = nullptr; s->scratch_bytes = 0;
         nups_status rc = nups_dev_alloc(s, (void**)&s->scratch, want);
