@@ -642,6 +642,9 @@ extern "C" nups_status nups_pull(nups_store* s, const uint32_t* d_keys, uint64_t
 // against four rows and three blocks (80 registers), the extra warps are worth more than the deeper unrolling at every skew
 // (1M keys x 128 floats: 275 vs 279 us at s = 0, 195 vs 199 us at s = 1.0 with 1,000 replicated keys, 138 vs 152 us at s = 1.4).
 constexpr int PUSH_UNROLL = 2;
+// 8-byte values: elements of two rows that a lane has in flight per table.  A small call is bound by the latency of these loads:
+// 20,000 rows of 100 values 30.8 us with two, 27.2 with four.
+constexpr int PUSH_WIDE = 4;
 constexpr int PUSH_THREADS = 256;
 constexpr int PUSH_BLOCKS = 4;            // one table; calls that update two tables at once keep three (80 registers)
 
@@ -808,12 +811,12 @@ push_atomic_kernel(View v, const uint32_t* __restrict__ keys, uint64_t n, PushPa
                 // them to the next one
                 static_assert(PUSH_UNROLL == 2, "two rows share a run of lanes");
                 const uint32_t both = src[1] >= 0 ? 2 * LE : LE;
-                for (uint32_t e0 = lane; e0 < both; e0 += 64) {
-                    typename E::T a[2], b[2];
-                    uint32_t c[2];
-                    bool second[2];
+                for (uint32_t e0 = lane; e0 < both; e0 += 32 * PUSH_WIDE) {
+                    typename E::T a[PUSH_WIDE], b[PUSH_WIDE];
+                    uint32_t c[PUSH_WIDE];
+                    bool second[PUSH_WIDE];
 #pragma unroll
-                    for (int k = 0; k < 2; ++k) {
+                    for (int k = 0; k < PUSH_WIDE; ++k) {
                         second[k] = e0 + 32 * k >= LE;
                         c[k] = e0 + 32 * k - (second[k] ? LE : 0u);
                         if (e0 + 32 * k < both) {
@@ -823,7 +826,7 @@ push_atomic_kernel(View v, const uint32_t* __restrict__ keys, uint64_t n, PushPa
                         }
                     }
 #pragma unroll
-                    for (int k = 0; k < 2; ++k) {
+                    for (int k = 0; k < PUSH_WIDE; ++k) {
                         if (e0 + 32 * k < both) {
                             const unsigned long long d = second[k] ? de[1] : de[0];
                             const bool h = HOT && (d & 1ull);
