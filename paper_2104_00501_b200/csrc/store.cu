@@ -1235,13 +1235,16 @@ push_chain_kernel(View v, const K* __restrict__ dest, const uint32_t* __restrict
 }
 
 // Few rows: every block works out all rows' destinations (into shared memory), a warp per row looks whether an earlier row
-// has the same destination and, if none has, finds the later ones by scanning, 32 rows at a step, and adds them in order.
-// One launch in place of seven; the scans grow with n^2.  Measured: 100 rows 15 us (72 us before), 3,000 rows of 64 floats
+// has the same destination and, if none has, finds the later ones by scanning, 128 rows at a step, and adds them in order;
+// the first of its rows and the stored row move towards L2 meanwhile.
+// One launch in place of seven; the scans grow with n^2.  Measured: 100 rows 15 us (72 us before), 3,000 rows of 64 floats pushed
+// and merged 22.9 us (29.2 with scans of 32 rows and nothing asked for ahead), 3,000 rows of 64 floats alone, before that,
 // 28 us, while the sort and what follows it take 37 us for 4,500 rows, and a frequent key's chain is slower here (2,500
 // rows, a third of them of one key: 73 us): the line lies at 3,072.
 constexpr uint32_t SMALL_PUSH_ROWS = 3072;
 constexpr unsigned SMALL_THREADS = 256, SMALL_LIST = 512;
 static_assert(SMALL_PUSH_ROWS <= 65536, "row numbers are kept in 16 bits");
+static_assert(SMALL_PUSH_ROWS % 128 == 0, "whole steps of the scans");
 
 template <bool HOT, bool F64>
 __global__ void __launch_bounds__(SMALL_THREADS)
@@ -1250,7 +1253,7 @@ push_small_kernel(PushDest<uint32_t, HOT> source, uint32_t n, const float4* __re
     grid_dependency_wait();
     constexpr unsigned FULL = 0xFFFFFFFFu;
     constexpr int U = 16;                                          // rows in flight
-    __shared__ uint32_t dest[SMALL_PUSH_ROWS];
+    __shared__ __align__(16) uint32_t dest[SMALL_PUSH_ROWS];
     __shared__ uint16_t list[SMALL_THREADS / 32][SMALL_LIST];
     const View& v = source.v;
     const uint32_t L4 = v.L4, invalid = source.invalid();
@@ -1263,31 +1266,44 @@ push_small_kernel(PushDest<uint32_t, HOT> source, uint32_t n, const float4* __re
         for (int m = 0; m < 4; ++m)
             if (b + threadIdx.x + m * SMALL_THREADS < n) dest[b + threadIdx.x + m * SMALL_THREADS] = d[m];
     }
+    if (threadIdx.x < (0u - n) % 128u) dest[n + threadIdx.x] = 0xFFFFFFFFu;         // up to a whole step: no destination
     __syncthreads();
+    const uint4* dest4 = reinterpret_cast<const uint4*>(dest);     // lane l of a step looks at rows 4 l ... 4 l + 3
     const uint32_t nwarps = gridDim.x * (SMALL_THREADS / 32);
     for (uint32_t i = (blockIdx.x * SMALL_THREADS + threadIdx.x) >> 5; i < n; i += nwarps) {
         const uint32_t d = dest[i];
         if (d == invalid) continue;
         bool first = true;
         for (uint32_t b = 0; b < i && first; b += 128) {
-            bool same = false;
-#pragma unroll
-            for (uint32_t k = 0; k < 4; ++k) {
-                const uint32_t j = b + 32 * k + lane;
-                same = same || (j < i && dest[j] == d);
-            }
-            first = !__any_sync(FULL, same);
+            const uint4 x = dest4[b / 4 + lane];
+            const uint32_t j = b + 4 * lane;
+            first = !__any_sync(FULL, (x.x == d && j < i) || (x.y == d && j + 1 < i) || (x.z == d && j + 2 < i) || (x.w == d && j + 3 < i));
         }
         if (!first) continue;
+        for (uint32_t c = 8 * lane; c < L4; c += 256) {
+            prefetch_l2(dv + (uint64_t)i * L4 + c);
+            prefetch_l2(dest_row<uint32_t>(v, d, 0) + c);
+            if (da) { prefetch_l2(da + (uint64_t)i * L4 + c); prefetch_l2(dest_row<uint32_t>(v, d, 1) + c); }
+        }
         // its rows, up to SMALL_LIST at a time
-        for (uint32_t b = i & ~31u; b < n;) {
+        for (uint32_t b = i & ~127u; b < n;) {
             uint32_t got = 0;
-            for (; b < n && got + 32 <= SMALL_LIST; b += 32) {
-                const uint32_t j = b + lane;
-                const bool member = j >= i && j < n && dest[j] == d;
-                const unsigned m = __ballot_sync(FULL, member);
-                if (member) list[wib][got + __popc(m & ((1u << lane) - 1u))] = (uint16_t)j;
-                got += __popc(m);
+            for (; b < n && got + 128 <= SMALL_LIST; b += 128) {
+                const uint4 x = dest4[b / 4 + lane];
+                const uint32_t j = b + 4 * lane;
+                // j + k < i: an earlier row, which the search above has shown to be another's
+                const unsigned mine = (x.x == d ? 1u : 0u) | (x.y == d ? 2u : 0u) | (x.z == d ? 4u : 0u) | (x.w == d ? 8u : 0u);
+                if (!__any_sync(FULL, mine != 0u)) continue;
+                uint32_t at = got;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const unsigned m = __ballot_sync(FULL, (mine >> k) & 1u);
+                    at += __popc(m & ((1u << lane) - 1u));
+                    got += __popc(m);
+                }
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    if ((mine >> k) & 1u) list[wib][at++] = (uint16_t)(j + k);
             }
             __syncwarp();
 #pragma unroll
