@@ -1402,193 +1402,309 @@ extern "C" nups_status nups_step_complex(nups_store* s, const uint32_t* d_h, con
 // ---------------------------------------------------------------------------------------------
 // matrix factorization over cells that come column by column (Section 5.1: every worker visits its cells
 // by column, to create locality in the accesses to column parameters).  Fast mode only.
-// A warp works on a stretch of consecutive cells.  The keys, cell values and replica slots of 32 cells are
-// loaded by the 32 lanes at once, one window ahead.  The rows of the row keys are fetched MF_RUN_DEPTH cells
-// ahead into a register ring.  The row of the column key stays in registers while the column stays the same
-// (the next column's row is fetched one cell before it is needed), and the column's update is summed in
-// registers and added once when the column changes: a column's row costs one read and one reduction per
-// stretch instead of one per cell.  Within a stretch the cells of a column all see the column's row from
-// before the stretch (the batch semantics of the deterministic mode); rows of row keys are read as they are.
+// A warp works on a stretch of consecutive cells.  The 32 lanes look up 32 cells at once (keys, slots, worker) and
+// leave where each cell's rows are read and updated in shared memory, so that a cell costs two shared-memory reads
+// instead of eight shuffles and the address arithmetic.  Cells are taken B at a time; the stored rows of the row
+// keys are fetched one batch ahead into registers, and the batch's scores are reduced together.
+// The stored row of the column key stays in registers while the column stays the same (the next column's row is on its
+// way from the moment the column before it begins), and the column's update is summed in registers and added once when
+// the column changes: a column's row costs one read and one reduction per stretch instead of one per cell.  Within
+// a stretch the cells of a column all see the column's stored row from before the stretch (the batch semantics of the
+// deterministic mode); rows of row keys are read as they are.  Columns that change inside a batch, keys out of range
+// between others and clipped updates take the cells of the batch one by one.
+// Bound by instruction issue and the latency of a warp's few cells: one cell at a time, with shuffled addresses and a
+// reduction of its own, took ~300 warp instructions.  65,536 cells: 100 floats 31.4 -> 20.3 us, 32 floats 27.2 -> 15.2;
+// 20,000 cells of 300 floats 40.1 -> 30.6.  (Replica rows read once per stretch instead of once per batch: 18.7 us, but the
+// step's loss moved by up to 4.5e-4, as cells no longer saw what others had just added.)
 // ---------------------------------------------------------------------------------------------
-constexpr int MF_RUN_DEPTH = 4;           // divides 32
 constexpr int MF_RUN_BLOCKS = 5;          // resident blocks per multiprocessor the grid is sized for
+
+struct MfRows { const float4* read; float4* add; };       // the stored row; the row that takes the update (nullptr: no cell)
 
 template <bool HOT, int CH, bool CLIP>
 __global__ void __launch_bounds__(128, MF_RUN_BLOCKS)
 mf_runs_kernel(View v, const uint32_t* __restrict__ rowk, const uint32_t* __restrict__ colk, const float* __restrict__ x,
                uint64_t n, float lr, float l2, float* __restrict__ loss_out)
 {
-    grid_dependency_wait();
     constexpr unsigned FULL = 0xFFFFFFFFu;
-    const unsigned lane = threadIdx.x & 31;
+    constexpr int B = CH == 1 ? 4 : 2;                     // cells per batch: what the registers hold twice over
+    constexpr unsigned BATCH = (1u << B) - 1;
+    constexpr bool AHEAD = CH <= 2;                        // fetch the next column's row ahead (longer rows: no registers left)
+    constexpr bool PENDING_AHEAD = HOT && CH == 1;         // ... and the pending updates of the next batch's replicated rows
+    __shared__ MfRows s_row[4][64], s_col[4][64];          // two windows of 32 cells per warp
+    __shared__ float s_x[4][64];
+    grid_dependency_wait();
+    const unsigned lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
     const uint32_t L4 = v.L4;
     const float4* val4 = (const float4*)v.val;
-    const float4* slab4 = (const float4*)v.dval;
-    double my_loss = 0.0;
+    float4* slab4 = (float4*)v.dval;
     const float bound = CLIP ? clip_bound(v) : 0.f;
     float my_clip = 0.f;
     unsigned my_clipped = 0;
-    const uint64_t stretch = (n + nwarps - 1) / nwarps;
+    // whole batches, unless that would leave warps without a cell in a small call
+    const uint64_t even = (n + nwarps - 1) / nwarps, stretch = even > B ? (even + B - 1) / B * B : even;
     const uint64_t first = warp * stretch < n ? warp * stretch : n;
     const uint64_t last = first + stretch < n ? first + stretch : n;            // this warp's cells: [first, last)
 
-    // one window = 32 consecutive cells, lane l holds cell l: keys (row key invalid when either key is),
-    // cell value, replica slots
-    struct Window { uint32_t ki, kj; float x; int si, sj; };
-    auto load_window = [&](uint64_t base) {
-        Window w = {NUPS_INVALID_KEY, NUPS_INVALID_KEY, 0.f, -1, -1};
+    // lane l's cell of a window: keys (both invalid when either is), value, slots.  Keys are loaded two windows ahead of
+    // the one at hand, slots one window ahead of where they are needed.
+    struct Cell { uint32_t ki, kj; float x; int si, sj; };
+    auto load_keys = [&](uint64_t base) {
+        Cell c = {NUPS_INVALID_KEY, NUPS_INVALID_KEY, 0.f, -1, -1};
         const uint64_t i = base + lane;
-        if (i < last) {
-            const uint32_t ki = rowk[i], kj = colk[i];
-            w.x = x[i];
-            if (ki < v.num_keys && kj < v.num_keys) {
-                w.ki = ki; w.kj = kj;
-                if (HOT) { w.si = __ldg(v.slot_of + ki); w.sj = __ldg(v.slot_of + kj); }
-            } else {
-                flag_bad_key(v);
-            }
+        if (i < last) { c.ki = rowk[i]; c.kj = colk[i]; c.x = x[i]; }
+        return c;
+    };
+    auto look_up = [&](Cell& c, uint64_t base) {
+        if (c.ki < v.num_keys && c.kj < v.num_keys) {
+            if (HOT) { c.si = __ldg(v.slot_of + c.ki); c.sj = __ldg(v.slot_of + c.kj); }
+        } else {
+            if (base + lane < last) flag_bad_key(v);
+            c.ki = c.kj = NUPS_INVALID_KEY;
         }
-        return w;
     };
-    Window cur = load_window(first), nxt = load_window(first + 32);
-    // cell t of the current window (t < 32) or of the next one (32 <= t < 64)
-    auto row_key_at = [&](uint32_t t) {
-        const uint32_t a = __shfl_sync(FULL, cur.ki, t & 31), b = __shfl_sync(FULL, nxt.ki, t & 31);
-        return t < 32 ? a : b;
+    auto stored_row = [&](uint32_t key) { return key != NUPS_INVALID_KEY ? val4 + (uint64_t)key * L4 : nullptr; };
+    struct Masks { unsigned ok, hot, turn; };              // cells to do, with a replicated row key, that change the column
+    float4* tail = nullptr;                                // column row of the last cell written down
+    auto write_down = [&](const Cell& c, uint64_t base, unsigned at) {
+        MfRows r = {stored_row(c.ki), nullptr}, h = {stored_row(c.kj), nullptr};
+        const bool ok = c.ki != NUPS_INVALID_KEY;
+        const uint32_t q = ok ? worker_of_item(base + lane, n, v.R) : 0u;
+        if (ok) {
+            r.add = HOT && c.si >= 0 ? slab4 + ((uint64_t)q * v.Hcap + (unsigned)c.si) * L4 : const_cast<float4*>(r.read);
+            h.add = HOT && c.sj >= 0 ? slab4 + ((uint64_t)q * v.Hcap + (unsigned)c.sj) * L4 : const_cast<float4*>(h.read);
+        }
+        s_row[wib][at + lane] = r;
+        s_col[wib][at + lane] = h;
+        s_x[wib][at + lane] = c.x;
+        float4* before = (float4*)__shfl_up_sync(FULL, (unsigned long long)h.add, 1);
+        if (lane == 0) before = tail;
+        tail = (float4*)__shfl_sync(FULL, (unsigned long long)h.add, 31);
+        Masks m;
+        m.ok = __ballot_sync(FULL, ok);
+        m.hot = HOT ? __ballot_sync(FULL, ok && c.si >= 0) : 0u;
+        m.turn = __ballot_sync(FULL, ok && h.add != before);
+        __syncwarp();
+        if (ok && (HOT || v.count || v.own)) {             // lane by lane, each for its own cell
+            if (HOT && c.si >= 0) mark_dirty(v, q, c.si);
+            if (HOT && c.sj >= 0 && h.add != before) mark_dirty(v, q, c.sj);
+            if (v.count) { note_access(v, c.ki, c.si, 2u); note_access(v, c.kj, c.sj, 2u); }
+            if (v.own) { mark_localize(v, c.ki, q); mark_localize(v, c.kj, q); }
+        }
+        return m;
     };
-    auto col_key_at = [&](uint32_t t) {
-        const uint32_t a = __shfl_sync(FULL, cur.kj, t & 31), b = __shfl_sync(FULL, nxt.kj, t & 31);
-        return t < 32 ? a : b;
-    };
-    auto fetch_row = [&](float4 (&dst)[CH], uint32_t key) {
+    // __ldcg: rows change while the kernel runs
+    auto fetch = [&](float4 (&dst)[CH], const float4* row) {
 #pragma unroll
         for (int m = 0; m < CH; ++m) {
             const uint32_t c = lane + 32 * m;
-            dst[m] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (key != NUPS_INVALID_KEY && c < L4) dst[m] = val4[(uint64_t)key * L4 + c];
+            dst[m] = c < L4 ? __ldcg(row + c) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
     };
 
-    float4 ring[MF_RUN_DEPTH][CH];                       // stored rows of the row keys of the next cells
+    Cell cell = load_keys(first), cell1 = load_keys(first + 32), cell2 = load_keys(first + 64);
+    look_up(cell, first);
+    look_up(cell1, first + 32);
+    unsigned at = 0;                                       // where the window at hand lies in the shared rows: 0 or 32
+    float4 w_next[B][CH];                                  // stored rows of the next batch's row keys
+    float4 p[HOT ? B : 1][CH];                             // pending updates of the replicated ones
+    auto fetch_batch = [&](uint32_t t, unsigned ok) {      // ok: this batch's bits
 #pragma unroll
-    for (int u = 0; u < MF_RUN_DEPTH; ++u) fetch_row(ring[u], row_key_at(u));
-    uint32_t h_key = NUPS_INVALID_KEY, h_next_key = NUPS_INVALID_KEY;
-    float4 h[CH], h_next[CH];                            // stored row of the current column, and of the one after it
-    {
-        const uint32_t k0 = col_key_at(0);
-        fetch_row(h_next, k0);
-        h_next_key = k0;
+        for (int u = 0; u < B; ++u)
+            if ((ok >> u) & 1) fetch(w_next[u], s_row[wib][(at + t + u) & 63].read);
+    };
+    auto fetch_pending = [&](uint32_t t, unsigned hot) {
+        if (!HOT || !hot) return;
+#pragma unroll
+        for (int u = 0; u < B; ++u)
+            if ((hot >> u) & 1) fetch(p[HOT ? u : 0], s_row[wib][(at + t + u) & 63].add);
+    };
+    // the first rows are on their way while the slots still are: a small call is nothing but these latencies
+    float4 h_next[AHEAD ? CH : 1];                         // the next column's stored row, on its way
+    const float4* next_row = nullptr;                      // the row h_next belongs to
+    s_row[wib][lane].read = stored_row(cell.ki);
+    __syncwarp();
+    fetch_batch(0, __ballot_sync(FULL, cell.ki != NUPS_INVALID_KEY) & BATCH);
+    if constexpr (AHEAD) {
+        next_row = stored_row(__shfl_sync(FULL, cell.kj, 0));
+        if (next_row) fetch(h_next, next_row);
     }
-    float* held_row = nullptr;                           // column row whose summed update is still in registers
-    float4 held[CH];
-    auto flush_held = [&]() {
+    __syncwarp();
+    Masks cur = write_down(cell, first, 0), nxt = {0u, 0u, 0u};
+    if (PENDING_AHEAD) fetch_pending(0, cur.hot & BATCH);
+
+    float4 h[CH], held[CH], hp[HOT ? CH : 1];              // the column's stored row, its summed update, its pending updates
+    float4* held_row = nullptr;                            // the row that takes the sum
+    bool hot_col = false;                                  // the column at hand is replicated: held_row is a replica row
+    const float rl = lr * l2;
+    auto flush = [&]() {
         if (!held_row) return;
 #pragma unroll
         for (int m = 0; m < CH; ++m) {
             const uint32_t c = lane + 32 * m;
-            if (c < L4) red_add_v4(held_row + 4 * c, held[m]);
+            if (c < L4) red_add_v4((float*)(held_row + c), held[m]);
         }
-        held_row = nullptr;
+    };
+    auto turn_to = [&](uint32_t t) {                       // make cell t's column the one at hand
+        const MfRows d = s_col[wib][(at + t) & 63];
+        if (d.add == held_row) return;
+        flush();
+        if constexpr (HOT) { if (d.add != d.read) fetch(hp, d.add); }
+        if (AHEAD && next_row == d.read) {
+#pragma unroll
+            for (int m = 0; m < CH; ++m) h[m] = h_next[AHEAD ? m : 0];
+        } else {
+            fetch(h, d.read);
+        }
+#pragma unroll
+        for (int m = 0; m < CH; ++m) held[m] = make_float4(0.f, 0.f, 0.f, 0.f);
+        held_row = d.add;
+        hot_col = HOT && d.add != d.read;
+        if constexpr (AHEAD) {
+            const unsigned later = t < 31 ? cur.turn & ~((2u << t) - 1) : 0u;
+            if (later) {
+                const MfRows e = s_col[wib][(at + __ffs(later) - 1) & 63];
+                fetch(h_next, e.read);
+                next_row = e.read;
+            }
+        }
     };
 
-    uint32_t q = worker_of_item(first < n ? first : 0, n, v.R);    // worker of the cell at hand, kept up as i grows
-    uint64_t q_end = worker_first_item(q + 1, n, v.R);
     float window_loss = 0.f;
+    double my_loss = 0.0;
     for (uint64_t base = first; base < last; base += 32) {
-        for (uint32_t t0 = 0; t0 < 32; t0 += MF_RUN_DEPTH) {
-            if (base + t0 >= last) break;
+        const uint32_t cells = (uint32_t)min((uint64_t)32, last - base);
+        if (base + 32 < last) {
+            nxt = write_down(cell1, base + 32, at ^ 32);
+            cell1 = cell2;
+            look_up(cell1, base + 64);
+            cell2 = load_keys(base + 96);
+        } else {
+            nxt.ok = nxt.hot = nxt.turn = 0u;
+        }
+        for (uint32_t t = 0; t < cells; t += B) {
+            float4 w[B][CH], hv[CH];                           // hv: the column's row with its pending updates
+            const unsigned ok = (cur.ok >> t) & BATCH, hot = (cur.hot >> t) & BATCH, turn = (cur.turn >> t) & BATCH;
+            if (!PENDING_AHEAD) fetch_pending(t, hot);
+            const bool one_column = !CLIP && (ok & (ok + 1u)) == 0u && (turn & ~1u) == 0u;   // ... and no cell missing between others
+            if (one_column && turn) turn_to(t);
 #pragma unroll
-            for (int u = 0; u < MF_RUN_DEPTH; ++u) {
-                const uint32_t t = t0 + u;
-                const uint64_t i = base + t;
-                if (i >= last) break;
-                const uint32_t ki = __shfl_sync(FULL, cur.ki, t), kj = __shfl_sync(FULL, cur.kj, t);
-                const float xv = __shfl_sync(FULL, cur.x, t);
-                const int si = __shfl_sync(FULL, cur.si, t), sj = __shfl_sync(FULL, cur.sj, t);
-                float4 w[CH];
+            for (int u = 0; u < B; ++u)
 #pragma unroll
-                for (int m = 0; m < CH; ++m) w[m] = ring[u][m];
-                fetch_row(ring[u], row_key_at(t + MF_RUN_DEPTH));
-                if (ki == NUPS_INVALID_KEY) continue;               // a bad key: flagged when the window was loaded
-                if (kj != h_key) {
-                    if (h_next_key != kj) { fetch_row(h_next, kj); h_next_key = kj; }
+                for (int m = 0; m < CH; ++m)
+                    w[u][m] = HOT && ((hot >> u) & 1) ? add4(w_next[u][m], p[HOT ? u : 0][m]) : w_next[u][m];
 #pragma unroll
-                    for (int m = 0; m < CH; ++m) h[m] = h_next[m];
-                    h_key = kj;
+            for (int m = 0; m < CH; ++m) hv[m] = hot_col ? add4(h[m], hp[HOT ? m : 0]) : h[m];
+            // pending updates are read again for every batch: replicated rows are those that other warps change most
+            fetch_batch(t + B, t + B < 32 ? (cur.ok >> (t + B)) & BATCH : nxt.ok & BATCH);
+            if (PENDING_AHEAD) fetch_pending(t + B, t + B < 32 ? (cur.hot >> (t + B)) & BATCH : nxt.hot & BATCH);
+            if constexpr (HOT) { if (one_column && hot_col) fetch(hp, held_row); }
+
+            if (one_column) {
+                float d[B];
+#pragma unroll
+                for (int u = 0; u < B; ++u) {
+                    d[u] = 0.f;
+#pragma unroll
+                    for (int m = 0; m < CH; ++m)
+                        d[u] += w[u][m].x * hv[m].x + w[u][m].y * hv[m].y + w[u][m].z * hv[m].z + w[u][m].w * hv[m].w;
                 }
+                // the scores together: after the halving steps lane l holds the score of cell l / (32 / B)
+                float y;
                 {
-                    const uint32_t kj1 = col_key_at(t + 1);
-                    if (kj1 != NUPS_INVALID_KEY && kj1 != h_key && kj1 != h_next_key) { fetch_row(h_next, kj1); h_next_key = kj1; }
+                    const bool up16 = (lane & 16) != 0;
+                    if constexpr (B == 4) {
+                        const bool up8 = (lane & 8) != 0;
+                        const float k0 = (up16 ? d[2] : d[0]) + __shfl_xor_sync(FULL, up16 ? d[0] : d[2], 16);
+                        const float k1 = (up16 ? d[3] : d[1]) + __shfl_xor_sync(FULL, up16 ? d[1] : d[3], 16);
+                        y = (up8 ? k1 : k0) + __shfl_xor_sync(FULL, up8 ? k0 : k1, 8);
+                    } else {
+                        y = (up16 ? d[1] : d[0]) + __shfl_xor_sync(FULL, up16 ? d[0] : d[1], 16);
+                        y += __shfl_xor_sync(FULL, y, 8);
+                    }
+                    y += __shfl_xor_sync(FULL, y, 4);
+                    y += __shfl_xor_sync(FULL, y, 2);
+                    y += __shfl_xor_sync(FULL, y, 1);
                 }
-                while (i >= q_end) q_end = worker_first_item(++q + 1, n, v.R);
-                const uint64_t pw = si >= 0 ? ((uint64_t)q * v.Hcap + (unsigned)si) * L4 : 0;
-                const uint64_t ph = sj >= 0 ? ((uint64_t)q * v.Hcap + (unsigned)sj) * L4 : 0;
-                float4 hv[CH];
+                const unsigned mine = lane / (32 / B);
+                const float err_l = s_x[wib][(at + t + mine) & 63] - y;
+                if (lane % (32 / B) == 0 && ((ok >> mine) & 1)) window_loss += err_l * err_l;
+                const float step_l = lr * err_l;
+#pragma unroll
+                for (int u = 0; u < B; ++u) {
+                    const float e = __shfl_sync(FULL, step_l, u * (32 / B));
+                    if (!((ok >> u) & 1)) continue;
+                    float4* const add = s_row[wib][(at + t + u) & 63].add;
+#pragma unroll
+                    for (int m = 0; m < CH; ++m) {
+                        const uint32_t c = lane + 32 * m;
+                        if (c < L4)
+                            red_add_v4((float*)(add + c), make_float4(e * hv[m].x - rl * w[u][m].x, e * hv[m].y - rl * w[u][m].y,
+                                                                      e * hv[m].z - rl * w[u][m].z, e * hv[m].w - rl * w[u][m].w));
+                        held[m].x += e * w[u][m].x; held[m].y += e * w[u][m].y;
+                        held[m].z += e * w[u][m].z; held[m].w += e * w[u][m].w;
+                    }
+                }
+                const float k = rl * (float)__popc(ok);
+#pragma unroll
+                for (int m = 0; m < CH; ++m) {
+                    held[m].x -= k * hv[m].x; held[m].y -= k * hv[m].y; held[m].z -= k * hv[m].z; held[m].w -= k * hv[m].w;
+                }
+                continue;
+            }
+#pragma unroll
+            for (int u = 0; u < B; ++u) {
+                if (!((ok >> u) & 1)) continue;                  // past the stretch, or a bad key (flagged at the lookup)
+                if ((turn >> u) & 1) turn_to(t + u);
+                float4* const add = s_row[wib][(at + t + u) & 63].add;
+                if constexpr (HOT) { if (hot_col) fetch(hp, held_row); }
                 float dot = 0.f;
 #pragma unroll
                 for (int m = 0; m < CH; ++m) {
-                    const uint32_t c = lane + 32 * m;
-                    hv[m] = h[m];
-                    if (c < L4) {
-                        if (HOT && si >= 0) w[m] = add4(w[m], slab4[pw + c]);       // the worker's pending replica updates
-                        if (HOT && sj >= 0) hv[m] = add4(hv[m], slab4[ph + c]);
-                    }
-                    dot += w[m].x * hv[m].x + w[m].y * hv[m].y + w[m].z * hv[m].z + w[m].w * hv[m].w;
+                    hv[m] = hot_col ? add4(h[m], hp[HOT ? m : 0]) : h[m];
+                    dot += w[u][m].x * hv[m].x + w[u][m].y * hv[m].y + w[u][m].z * hv[m].z + w[u][m].w * hv[m].w;
                 }
-                const float err = xv - warp_sum(dot);
-                float fw = lr, fh = lr;                                 // learning rate times the clipping factor
-                if (CLIP && (si >= 0 || sj >= 0)) {
+                const float err = s_x[wib][(at + t + u) & 63] - warp_sum(dot);
+                float fw = lr, fh = lr;                          // learning rate times the clipping factor
+                if (CLIP && (((hot >> u) & 1) || hot_col)) {
                     float nw2 = 0.f, nh2 = 0.f;
 #pragma unroll
                     for (int m = 0; m < CH; ++m) {
-                        if (lane + 32 * m < L4) {
-                            const float4 a = make_float4(err * hv[m].x - l2 * w[m].x, err * hv[m].y - l2 * w[m].y,
-                                                         err * hv[m].z - l2 * w[m].z, err * hv[m].w - l2 * w[m].w);
-                            const float4 b = make_float4(err * w[m].x - l2 * hv[m].x, err * w[m].y - l2 * hv[m].y,
-                                                         err * w[m].z - l2 * hv[m].z, err * w[m].w - l2 * hv[m].w);
-                            nw2 += a.x * a.x + a.y * a.y + a.z * a.z + a.w * a.w;
-                            nh2 += b.x * b.x + b.y * b.y + b.z * b.z + b.w * b.w;
-                        }
+                        const float4 a = make_float4(err * hv[m].x - l2 * w[u][m].x, err * hv[m].y - l2 * w[u][m].y,
+                                                     err * hv[m].z - l2 * w[u][m].z, err * hv[m].w - l2 * w[u][m].w);
+                        const float4 b = make_float4(err * w[u][m].x - l2 * hv[m].x, err * w[u][m].y - l2 * hv[m].y,
+                                                     err * w[u][m].z - l2 * hv[m].z, err * w[u][m].w - l2 * hv[m].w);
+                        nw2 += a.x * a.x + a.y * a.y + a.z * a.z + a.w * a.w;
+                        nh2 += b.x * b.x + b.y * b.y + b.z * b.z + b.w * b.w;
                     }
                     float applied = 0.f, f;
-                    if (si >= 0) { applied += clip_norm(lr * sqrtf(warp_sum(nw2)), bound, &f); fw = lr * f; }
-                    if (sj >= 0) { applied += clip_norm(lr * sqrtf(warp_sum(nh2)), bound, &f); fh = lr * f; }
+                    if ((hot >> u) & 1) { applied += clip_norm(lr * sqrtf(warp_sum(nw2)), bound, &f); fw = lr * f; }
+                    if (hot_col) { applied += clip_norm(lr * sqrtf(warp_sum(nh2)), bound, &f); fh = lr * f; }
                     my_clip += applied;
-                    my_clipped += (si >= 0 ? 1u : 0u) + (sj >= 0 ? 1u : 0u);
+                    my_clipped += ((hot >> u) & 1) + (hot_col ? 1u : 0u);
                 }
-                float* ow = si >= 0 ? v.dval + pw * 4 : v.val + (uint64_t)ki * L4 * 4;
-                float* oh = sj >= 0 ? v.dval + ph * 4 : v.val + (uint64_t)kj * L4 * 4;
-                if (held_row != oh) flush_held();
 #pragma unroll
                 for (int m = 0; m < CH; ++m) {
                     const uint32_t c = lane + 32 * m;
-                    if (c < L4) {
-                        const float4 dw = make_float4(fw * (err * hv[m].x - l2 * w[m].x), fw * (err * hv[m].y - l2 * w[m].y),
-                                                      fw * (err * hv[m].z - l2 * w[m].z), fw * (err * hv[m].w - l2 * w[m].w));
-                        const float4 dh = make_float4(fh * (err * w[m].x - l2 * hv[m].x), fh * (err * w[m].y - l2 * hv[m].y),
-                                                      fh * (err * w[m].z - l2 * hv[m].z), fh * (err * w[m].w - l2 * hv[m].w));
-                        red_add_v4(ow + 4 * c, dw);
-                        held[m] = oh == held_row ? add4(held[m], dh) : dh;
-                    }
+                    if (c < L4)
+                        red_add_v4((float*)(add + c), make_float4(fw * (err * hv[m].x - l2 * w[u][m].x), fw * (err * hv[m].y - l2 * w[u][m].y),
+                                                                  fw * (err * hv[m].z - l2 * w[u][m].z), fw * (err * hv[m].w - l2 * w[u][m].w)));
+                    held[m] = add4(held[m], make_float4(fh * (err * w[u][m].x - l2 * hv[m].x), fh * (err * w[u][m].y - l2 * hv[m].y),
+                                                        fh * (err * w[u][m].z - l2 * hv[m].z), fh * (err * w[u][m].w - l2 * hv[m].w)));
                 }
-                held_row = oh;
-                if (lane == 0) {
-                    if (si >= 0) mark_dirty(v, q, si);
-                    if (sj >= 0) mark_dirty(v, q, sj);
-                    if (v.count) { note_access(v, ki, si, 2u); note_access(v, kj, sj, 2u); }
-                    if (v.own) { mark_localize(v, ki, q); mark_localize(v, kj, q); }
-                }
-                window_loss += err * err;
+                if (lane == 0) window_loss += err * err;
             }
         }
         my_loss += (double)window_loss;
         window_loss = 0.f;
         cur = nxt;
-        nxt = load_window(base + 64);
+        at ^= 32;
     }
-    flush_held();
+    flush();
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) my_loss += __shfl_xor_sync(FULL, my_loss, o);
     loss_finish(v, my_loss, n, loss_out);
     if (CLIP) clip_finish(v, (double)my_clip, my_clipped);
 }
@@ -1680,7 +1796,9 @@ static nups_status mf_step(nups_store* s, const uint32_t* d_row, const uint32_t*
     rc = step_buffers(s, n, 2, false, &b);
     if (rc != NUPS_OK) return rc;
     View v = nups_view(s);
-    const bool by_column = cells_by_column && !s->cfg.deterministic;    // the ordered mode is the same for any order
+    // The ordered mode is the same for any order.  A call with a cell per resident warp at most has no runs to save on, and the
+    // plain kernel has less to set up: 1,935 cells of 64 floats 5.9 us, 6.6 with the kernel for runs (65,536 cells: 102 and 20).
+    const bool by_column = cells_by_column && !s->cfg.deterministic && n > (uint64_t)s->sm_count * MF_RUN_BLOCKS * 4;
     nups_time_begin(s, st, NUPS_TIMED_STEP);
     if (s->vb == 8) {
         const unsigned grid = step_grid(s, n, 8);

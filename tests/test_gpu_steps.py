@@ -459,3 +459,32 @@ def test_fast_mode_with_clipping_tracks_the_clipped_oracle():
     assert cs == co and ss == pytest.approx(so, rel=0.1)
     assert s.status_check() == 0
     s.close()
+
+
+@pytest.mark.parametrize("runs", [False, True])
+@pytest.mark.parametrize("n,L", [(2960, 100), (2961, 100), (7003, 200), (24_001, 12), (9001, 512)])
+def test_mf_by_column_with_bad_keys_at_the_sizes_where_its_batches_change(n, L, runs):
+    # a warp's stretch of 1, 2, 3, 9 (rounded to whole batches) and 4 cells, more than 32 with many cells; runs of one
+    # column and columns that change at every cell; keys out of range inside a batch: those cells change nothing
+    M, N, R = 3000, 900, 3
+    i, j, x = inputs.mf_cells(n, M, N, 0.3, 8, 0.1, 2, by_column_of=20 * n if runs else 0)
+    i, j, x = inputs.u32(i), inputs.u32(j), x.numpy()
+    bad = np.random.default_rng(n).random(n) < 0.02
+    init = np.random.default_rng(3).normal(0, 0.3, size=(M + N, L)).astype(np.float32)
+    o, s = make_pair(M + N, L, R=R, init=init, deterministic=False)
+    hot = np.unique(np.concatenate([i[:20], j[:20]])).astype(np.uint32)
+    o.set_management(hot, REPLICATE)
+    s.set_management(dev_keys(hot), REPLICATE)
+    lr = 2e-6                                  # tiny, see test_mf_fast_mode_on_cells_in_column_order
+    bi = i.copy()
+    bi[bad] = M + N + 7
+    s.step_mf(dev_keys(bi), dev_keys(j), dev_f32(x), lr, 0.01, loss_buf(), by_column=True)
+    assert s.status_check() == -4
+    o.step_mf(bi, j, x, lr, 0.01)
+    o.sync()
+    s.sync()
+    d_o = o.table(0).astype(np.float64) - init
+    d_s = s.read_table(0).cpu().numpy().astype(np.float64) - init
+    norm = np.linalg.norm(d_o, axis=1)
+    assert np.all(np.linalg.norm(d_s - d_o, axis=1) <= 0.01 * norm + 2e-6 * np.sqrt(L / 100 + 1))   # fp32 rounding of every stored value
+    assert norm.max() > 2e-5
