@@ -116,3 +116,9 @@ def test_more_destinations_than_32_bits_number(n):
         assert np.array_equal(row, halves[0] if len(halves) == 1 else halves[0] + halves[1]), k
     assert s.status_check() == -4
     s.close()
+
+
+@pytest.mark.parametrize("kind", ["skewed", "one", "bad"])
+@pytest.mark.parametrize("n,L", [(127, 36), (128, 4), (129, 64), (641, 8)])
+def test_small_pushes_at_whole_steps_of_the_scans(n, L, kind):
+    test_every_size_matches_the_oracle_bit_for_bit(n, L, kind, 90)
