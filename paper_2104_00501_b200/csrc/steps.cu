@@ -1476,6 +1476,7 @@ mf_runs_kernel(View v, const uint32_t* __restrict__ rowk, const uint32_t* __rest
             r.add = HOT && c.si >= 0 ? slab4 + ((uint64_t)q * v.Hcap + (unsigned)c.si) * L4 : const_cast<float4*>(r.read);
             h.add = HOT && c.sj >= 0 ? slab4 + ((uint64_t)q * v.Hcap + (unsigned)c.sj) * L4 : const_cast<float4*>(h.read);
         }
+        __syncwarp();                                      // the window that lay here has been read by every lane
         s_row[wib][at + lane] = r;
         s_col[wib][at + lane] = h;
         s_x[wib][at + lane] = c.x;
@@ -1531,7 +1532,6 @@ mf_runs_kernel(View v, const uint32_t* __restrict__ rowk, const uint32_t* __rest
         next_row = stored_row(__shfl_sync(FULL, cell.kj, 0));
         if (next_row) fetch(h_next, next_row);
     }
-    __syncwarp();
     Masks cur = write_down(cell, first, 0), nxt = {0u, 0u, 0u};
     if (PENDING_AHEAD) fetch_pending(0, cur.hot & BATCH);
 

@@ -241,6 +241,54 @@ def test_mf_by_column_matches_the_oracle_at_a_normal_learning_rate_where_cells_c
     assert s.status_check() == 0
 
 
+def _stretch_of_the_runs(n, L):
+    """Cells per warp and warps of the kernel for runs: whole batches of four cells (two for rows of more than 128 floats)."""
+    even, warps = _by_column_stretch(n)
+    batch = 4 if L <= 128 else 2
+    return (-(-even // batch) * batch if even > batch else even), warps
+
+
+@pytest.mark.parametrize("hot", [False, True])
+@pytest.mark.parametrize("per_warp,L", [(7, 100), (33, 8), (36, 100), (68, 12), (70, 132), (101, 8), (68, 260)])
+def test_mf_by_column_over_several_windows_of_cells(per_warp, L, hot):
+    # a warp takes its stretch in windows of 32 cells.  No two cells share a row key and a column's cells lie in one stretch and
+    # follow one another, so the oracle's batch step is what the kernel computes, at a normal learning rate; columns begin and end
+    # before, at and after the windows' ends, and cells with a key out of range lie between them
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    n = sms * 5 * 4 * per_warp
+    stretch, warps = _stretch_of_the_runs(n, L)
+    rng = np.random.default_rng(per_warp)
+    first_cells = [0, 1, 5, 31, 32, 33, 40, 63, 64, 66, 95, 96, 97]             # of columns, in even stretches; random ones in odd
+    begins = np.zeros(n, bool)
+    for w in range(warps):
+        here = np.array(first_cells) if w % 2 == 0 else np.flatnonzero(rng.random(stretch) < rng.choice([0.03, 0.3, 0.9]))
+        cells = w * stretch + np.append(here, 0)
+        begins[cells[(cells < n) & (cells < (w + 1) * stretch)]] = True
+    M, N, R = n, int(begins.sum()), 3                                           # R: workers change inside stretches
+    i = rng.permutation(M).astype(np.uint32)
+    j = (M + rng.permutation(N)[np.cumsum(begins) - 1]).astype(np.uint32)
+    x = rng.normal(0, 1, n).astype(np.float32)
+    bad = (rng.random(n) < 0.03) | (np.arange(n) % (5 * stretch) < 3)           # ... among them whole beginnings of stretches
+    o, s = make_pair(M + N, L, R=R, deterministic=False, sync_interval=1)
+    o.init_uniform(0, 4, 0.3)
+    s.init_uniform(0, 4, 0.3)
+    if hot:
+        keys = np.concatenate([rng.choice(i, 3000, replace=False), rng.choice(np.unique(j), min(N, 3000) // 2, replace=False)])
+        o.set_management(keys, REPLICATE)
+        s.set_management(dev_keys(keys), REPLICATE)
+    start = o.table(0).copy()
+    which = rng.random(n) < 0.5
+    i[bad & which] = M + N + 7
+    j[bad & ~which] = 0xFFFFFFF0
+    lb = loss_buf()
+    lo = o.step_mf(i, j, x, 0.01, 0.01)
+    s.step_mf(dev_keys(i), dev_keys(j), dev_f32(x), 0.01, 0.01, lb, by_column=True)
+    assert abs(lb.item() - lo) <= 1e-5 * abs(lo)
+    np.testing.assert_allclose(s.read_table(0).cpu().numpy(), o.table(0), rtol=RTOL, atol=ATOL)
+    assert np.abs(o.table(0) - start).max() > 1e-3
+    assert s.status_check() == -4
+
+
 @pytest.mark.parametrize("L,n_centres,hot_n", [(300, 1900, 60), (64, 333, 0), (512, 700, 30), (12, 257, 10)])
 def test_sgns_fast_mode_one_step_with_runs_of_one_centre_word(L, n_centres, hot_n):
     # pairs arrive centre by centre (10 context positions per centre position): the fast kernel reads a centre's row
