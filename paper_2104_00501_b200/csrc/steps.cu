@@ -1564,10 +1564,10 @@ mf_runs_kernel(View v, const uint32_t* __restrict__ rowk, const uint32_t* __rest
         hot_col = HOT && d.add != d.read;
         if constexpr (AHEAD) {
             const unsigned later = t < 31 ? cur.turn & ~((2u << t) - 1) : 0u;
+            next_row = nullptr;                            // used up: were it kept, the row would come back as it was
             if (later) {
-                const MfRows e = s_col[wib][(at + __ffs(later) - 1) & 63];
-                fetch(h_next, e.read);
-                next_row = e.read;
+                next_row = s_col[wib][(at + __ffs(later) - 1) & 63].read;
+                fetch(h_next, next_row);
             }
         }
     };

@@ -289,6 +289,32 @@ def test_mf_by_column_over_several_windows_of_cells(per_warp, L, hot):
     assert s.status_check() == -4
 
 
+@pytest.mark.parametrize("L", [8, 132])
+def test_mf_by_column_a_column_that_comes_back_shows_what_the_stretch_added_to_it(L):
+    # a stretch of three windows: a first column, a second one to the window's end, a third for a window, the second one again.
+    # Its row has been read ahead twice by then; the cells of its second turn see it with the updates of its first
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    stretch = 96
+    n = sms * 5 * 4 * stretch
+    assert _stretch_of_the_runs(n, L) == (stretch, n // stretch)
+    M, N = n, 3 * (n // stretch)
+    rng = np.random.default_rng(9)
+    i = rng.permutation(M).astype(np.uint32)
+    column = np.repeat([0, 1, 2, 1], [1, 31, 32, 32])
+    j = (M + rng.permutation(N)[(3 * np.arange(n // stretch)[:, None] + column).reshape(-1)]).astype(np.uint32)
+    x = rng.normal(0, 1, n).astype(np.float32)
+    o, s = make_pair(M + N, L, deterministic=False, sync_interval=1)
+    o.init_uniform(0, 4, 0.3)
+    s.init_uniform(0, 4, 0.3)
+    again = np.tile(np.arange(stretch) >= 64, n // stretch)
+    lo = [o.step_mf(np.ascontiguousarray(i[part]), np.ascontiguousarray(j[part]), np.ascontiguousarray(x[part]), 0.01, 0.01) for part in (~again, again)]
+    lb = loss_buf()
+    s.step_mf(dev_keys(i), dev_keys(j), dev_f32(x), 0.01, 0.01, lb, by_column=True)
+    want = (2 * lo[0] + lo[1]) / 3
+    assert abs(lb.item() - want) <= 1e-5 * abs(want)
+    np.testing.assert_allclose(s.read_table(0).cpu().numpy(), o.table(0), rtol=RTOL, atol=ATOL)
+
+
 @pytest.mark.parametrize("L,n_centres,hot_n", [(300, 1900, 60), (64, 333, 0), (512, 700, 30), (12, 257, 10)])
 def test_sgns_fast_mode_one_step_with_runs_of_one_centre_word(L, n_centres, hot_n):
     # pairs arrive centre by centre (10 context positions per centre position): the fast kernel reads a centre's row
