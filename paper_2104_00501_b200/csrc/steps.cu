@@ -1410,12 +1410,15 @@ extern "C" nups_status nups_step_complex(nups_store* s, const uint32_t* d_h, con
 // way from the moment the column before it begins), and the column's update is summed in registers and added once when
 // the column changes: a column's row costs one read and one reduction per stretch instead of one per cell.  Within
 // a stretch the cells of a column all see the column's stored row from before the stretch (the batch semantics of the
-// deterministic mode); rows of row keys are read as they are.  Columns that change inside a batch, keys out of range
+// deterministic mode); rows of row keys are read as they are, stored rows while the batch before is at work and pending updates of
+// replicated rows, of row and column keys, when the batch begins.  Columns that change inside a batch, keys out of range
 // between others and clipped updates take the cells of the batch one by one.
 // Bound by instruction issue and the latency of a warp's few cells: one cell at a time, with shuffled addresses and a
 // reduction of its own, took ~300 warp instructions.  65,536 cells: 100 floats 31.4 -> 20.3 us, 32 floats 27.2 -> 15.2;
-// 20,000 cells of 300 floats 40.1 -> 30.6.  (Replica rows read once per stretch instead of once per batch: 18.7 us, but the
-// step's loss moved by up to 4.5e-4, as cells no longer saw what others had just added.)
+// 20,000 cells of 300 floats 40.1 -> 30.6.  What other cells see of one another's updates moves the step's loss: against one
+// cell at a time, by 1.2e-5 of it at 65,536 cells of 100 floats and 6.5e-5 at 20,000 (2.3e-5 and 1.1e-4 when the pending updates
+// were read a batch ahead, which was no faster for rows of at most 256 floats and 4 to 6 % faster for longer ones; 4.5e-4 when
+// they were read once per stretch, 18.7 us).
 // ---------------------------------------------------------------------------------------------
 constexpr int MF_RUN_BLOCKS = 5;          // resident blocks per multiprocessor the grid is sized for
 
@@ -1430,7 +1433,6 @@ mf_runs_kernel(View v, const uint32_t* __restrict__ rowk, const uint32_t* __rest
     constexpr int B = CH == 1 ? 4 : 2;                     // cells per batch: what the registers hold twice over
     constexpr unsigned BATCH = (1u << B) - 1;
     constexpr bool AHEAD = CH <= 2;                        // fetch the next column's row ahead (longer rows: no registers left)
-    constexpr bool PENDING_AHEAD = HOT && CH == 1;         // ... and the pending updates of the next batch's replicated rows
     __shared__ MfRows s_row[4][64], s_col[4][64];          // two windows of 32 cells per warp
     __shared__ float s_x[4][64];
     grid_dependency_wait();
@@ -1533,7 +1535,6 @@ mf_runs_kernel(View v, const uint32_t* __restrict__ rowk, const uint32_t* __rest
         if (next_row) fetch(h_next, next_row);
     }
     Masks cur = write_down(cell, first, 0), nxt = {0u, 0u, 0u};
-    if (PENDING_AHEAD) fetch_pending(0, cur.hot & BATCH);
 
     float4 h[CH], held[CH], hp[HOT ? CH : 1];              // the column's stored row, its summed update, its pending updates
     float4* held_row = nullptr;                            // the row that takes the sum
@@ -1551,7 +1552,6 @@ mf_runs_kernel(View v, const uint32_t* __restrict__ rowk, const uint32_t* __rest
         const MfRows d = s_col[wib][(at + t) & 63];
         if (d.add == held_row) return;
         flush();
-        if constexpr (HOT) { if (d.add != d.read) fetch(hp, d.add); }
         if (AHEAD && next_row == d.read) {
 #pragma unroll
             for (int m = 0; m < CH; ++m) h[m] = h_next[AHEAD ? m : 0];
@@ -1587,9 +1587,11 @@ mf_runs_kernel(View v, const uint32_t* __restrict__ rowk, const uint32_t* __rest
         for (uint32_t t = 0; t < cells; t += B) {
             float4 w[B][CH], hv[CH];                           // hv: the column's row with its pending updates
             const unsigned ok = (cur.ok >> t) & BATCH, hot = (cur.hot >> t) & BATCH, turn = (cur.turn >> t) & BATCH;
-            if (!PENDING_AHEAD) fetch_pending(t, hot);
+            // pending updates are read when the batch begins and not ahead: replicated rows are those that other warps change most
+            fetch_pending(t, hot);
             const bool one_column = !CLIP && (ok & (ok + 1u)) == 0u && (turn & ~1u) == 0u;   // ... and no cell missing between others
             if (one_column && turn) turn_to(t);
+            if constexpr (HOT) { if (one_column && hot_col) fetch(hp, held_row); }
 #pragma unroll
             for (int u = 0; u < B; ++u)
 #pragma unroll
@@ -1597,10 +1599,7 @@ mf_runs_kernel(View v, const uint32_t* __restrict__ rowk, const uint32_t* __rest
                     w[u][m] = HOT && ((hot >> u) & 1) ? add4(w_next[u][m], p[HOT ? u : 0][m]) : w_next[u][m];
 #pragma unroll
             for (int m = 0; m < CH; ++m) hv[m] = hot_col ? add4(h[m], hp[HOT ? m : 0]) : h[m];
-            // pending updates are read again for every batch: replicated rows are those that other warps change most
             fetch_batch(t + B, t + B < 32 ? (cur.ok >> (t + B)) & BATCH : nxt.ok & BATCH);
-            if (PENDING_AHEAD) fetch_pending(t + B, t + B < 32 ? (cur.hot >> (t + B)) & BATCH : nxt.hot & BATCH);
-            if constexpr (HOT) { if (one_column && hot_col) fetch(hp, held_row); }
 
             if (one_column) {
                 float d[B];

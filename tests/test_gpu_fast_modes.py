@@ -315,6 +315,41 @@ def test_mf_by_column_a_column_that_comes_back_shows_what_the_stretch_added_to_i
     np.testing.assert_allclose(s.read_table(0).cpu().numpy(), o.table(0), rtol=RTOL, atol=ATOL)
 
 
+@pytest.mark.parametrize("L", [100, 200, 260])
+def test_mf_by_column_a_batch_of_cells_sees_the_replica_updates_of_the_batch_before(L):
+    # replicas hold the rows that change most, so what a batch reads of them is as it is when the batch begins.  A warp's own
+    # updates show it: a replicated row key once in every batch, and the column itself as the row key of the first batch's last cell
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    W, stretch, lr, l2 = sms * 5 * 4, 40, 0.05, 0.01
+    batch, n = 4 if L <= 128 else 2, W * stretch
+    assert _stretch_of_the_runs(n, L) == (stretch, W)
+    rng = np.random.default_rng(11)
+    keys = rng.permutation(n + 2 * W).astype(np.uint32)
+    row, col, own = keys[:n].reshape(W, stretch).copy(), keys[n:n + W], keys[n + W:]
+    row[:, ::batch] = own[:, None]
+    row[:, batch - 1] = col
+    x = rng.normal(0, 1, (W, stretch)).astype(np.float32)
+    o, s = make_pair(n + 2 * W, L, deterministic=False, sync_interval=1)
+    o.init_uniform(0, 4, 0.3)
+    s.init_uniform(0, 4, 0.3)
+    hot = keys[n:]
+    s.set_management(dev_keys(hot), REPLICATE)
+    lb = loss_buf()
+    s.step_mf(dev_keys(row.reshape(-1)), dev_keys(np.repeat(col, stretch)), dev_f32(x.reshape(-1)), lr, l2, lb, by_column=True)
+    want, total = o.table(0).astype(np.float64), 0.0
+    stored, held = want[col], np.zeros((W, L))
+    for b in range(0, stretch, batch):
+        h, w = want[col], want[row[:, b:b + batch]]                    # in `want` a replicated row is the stored one and its replica's
+        err = x[:, b:b + batch] - np.einsum("wbl,wl->wb", w, h)
+        total += (err ** 2).sum()
+        held += lr * (np.einsum("wb,wbl->wl", err, w) - batch * l2 * h)
+        np.add.at(want, row[:, b:b + batch], lr * (err[..., None] * h[:, None] - l2 * w))
+    want[col] += held
+    assert np.abs(want[col] - stored).max() > 0.1
+    assert abs(lb.item() - total / n) <= 1e-5 * total / n
+    np.testing.assert_allclose(s.read_table(0).cpu().numpy(), want, rtol=RTOL, atol=ATOL)
+
+
 @pytest.mark.parametrize("L,n_centres,hot_n", [(300, 1900, 60), (64, 333, 0), (512, 700, 30), (12, 257, 10)])
 def test_sgns_fast_mode_one_step_with_runs_of_one_centre_word(L, n_centres, hot_n):
     # pairs arrive centre by centre (10 context positions per centre position): the fast kernel reads a centre's row
