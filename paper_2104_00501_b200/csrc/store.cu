@@ -1281,8 +1281,7 @@ push_small_kernel(PushDest<uint32_t, HOT> source, uint32_t n, const float4* __re
         }
         if (!first) continue;
         for (uint32_t c = 8 * lane; c < L4; c += 256) {
-            prefetch_l2(dv + (uint64_t)i * L4 + c);
-            prefetch_l2(dest_row<uint32_t>(v, d, 0) + c);
+            if (dv) { prefetch_l2(dv + (uint64_t)i * L4 + c); prefetch_l2(dest_row<uint32_t>(v, d, 0) + c); }
             if (da) { prefetch_l2(da + (uint64_t)i * L4 + c); prefetch_l2(dest_row<uint32_t>(v, d, 1) + c); }
         }
         // its rows, up to SMALL_LIST at a time

@@ -122,3 +122,30 @@ def test_more_destinations_than_32_bits_number(n):
 @pytest.mark.parametrize("n,L", [(127, 36), (128, 4), (129, 64), (641, 8)])
 def test_small_pushes_at_whole_steps_of_the_scans(n, L, kind):
     test_every_size_matches_the_oracle_bit_for_bit(n, L, kind, 90)
+
+
+@pytest.mark.parametrize("n", [1, 700, 3072, 9001])
+@pytest.mark.parametrize("value_bytes,L", [(4, 100), (8, 34)])
+def test_accumulators_alone(n, value_bytes, L):
+    # the value delta may be left out: the value table stays as it is
+    nk, R = 3000, 3
+    rng = np.random.default_rng(n)
+    real = np.float64 if value_bytes == 8 else np.float32
+    o = Oracle(nk, L, workers=R, with_adagrad=True, value_bytes=value_bytes)
+    s = binding.Store(nk, L, workers=R, with_adagrad=True, deterministic=True, value_bytes=value_bytes)
+    for which in (0, 1):
+        init = rng.normal(size=(nk, L)).astype(real)
+        o.table(which)[:] = init
+        s.write_table(which, init)
+    hot = np.arange(40, dtype=np.uint32)
+    o.set_management(hot, REPLICATE)
+    s.set_management(dev_keys(hot), binding.REPLICATE)
+    keys = (rng.zipf(1.3, n) % nk).astype(np.uint32)
+    da = rng.random((n, L)).astype(real)
+    o.push(keys, np.zeros((n, L), real), da)
+    s.push(dev_keys(keys), None, torch.from_numpy(da).cuda())
+    o.sync()
+    s.sync()
+    tables_equal(o, s, 0)
+    tables_equal(o, s, 1)
+    assert s.status_check() == 0
