@@ -643,8 +643,13 @@ extern "C" nups_status nups_pull(nups_store* s, const uint32_t* d_keys, uint64_t
 // (1M keys x 128 floats: 275 vs 279 us at s = 0, 195 vs 199 us at s = 1.0 with 1,000 replicated keys, 138 vs 152 us at s = 1.4).
 constexpr int PUSH_UNROLL = 2;
 // 8-byte values: elements of two rows that a lane has in flight per table.  A small call is bound by the latency of these loads:
-// 20,000 rows of 100 values 30.8 us with two, 27.2 with four.
+// 20,000 rows of 100 values 16.8 us with two, 14.1 with four; 300,000 rows of 128 values 153.6 and 151.0 us, 50,021 rows pushed to two
+// tables after a pull 101.6 and 92.4.  Two cover both rows where they have at most PUSH_SHORT values: 300,000 rows of 32 values take
+// 44.0 us with four, 41.3 with two.  Where warps share a window, a second form for short rows costs the longer ones more than it gives
+// (two tables: 50.7 -> 54.6 us for 20,000 rows of 100; 20,000 rows of 32 8.6 -> 7.8).  The two rows' offsets are worked out before the
+// loads: per element they took registers that had to be spilled (300,000 rows of 128 values, 500 keys replicated, 137.8 -> 134).
 constexpr int PUSH_WIDE = 4;
+constexpr uint32_t PUSH_SHORT = 32;
 constexpr int PUSH_THREADS = 256;
 constexpr int PUSH_BLOCKS = 4;            // one table; calls that update two tables at once keep three (80 registers)
 
@@ -811,31 +816,34 @@ push_atomic_kernel(View v, const uint32_t* __restrict__ keys, uint64_t n, PushPa
                 // them to the next one
                 static_assert(PUSH_UNROLL == 2, "two rows share a run of lanes");
                 const uint32_t both = src[1] >= 0 ? 2 * LE : LE;
-                for (uint32_t e0 = lane; e0 < both; e0 += 32 * PUSH_WIDE) {
-                    typename E::T a[PUSH_WIDE], b[PUSH_WIDE];
-                    uint32_t c[PUSH_WIDE];
-                    bool second[PUSH_WIDE];
+                // where element 0 of the run would lie if all of it were the first row's, or the second one's
+                const uint64_t from[2] = {(base + src[0]) * LE, (base + src[1]) * LE - LE};
+                auto turn = [&](uint32_t e0, auto width) {
+                    constexpr int W = decltype(width)::value;
+                    typename E::T a[W], b[W];
 #pragma unroll
-                    for (int k = 0; k < PUSH_WIDE; ++k) {
-                        second[k] = e0 + 32 * k >= LE;
-                        c[k] = e0 + 32 * k - (second[k] ? LE : 0u);
-                        if (e0 + 32 * k < both) {
-                            const uint64_t in_off = (base + (second[k] ? src[1] : src[0])) * LE + c[k];
+                    for (int k = 0; k < W; ++k) {
+                        const uint32_t e = e0 + 32 * k;
+                        if (e < both) {
+                            const uint64_t in_off = (e >= LE ? from[1] : from[0]) + e;
                             a[k] = E::load(A.delta, in_off);
                             if (TWO) b[k] = E::load(B.delta, in_off);
                         }
                     }
 #pragma unroll
-                    for (int k = 0; k < PUSH_WIDE; ++k) {
-                        if (e0 + 32 * k < both) {
-                            const unsigned long long d = second[k] ? de[1] : de[0];
+                    for (int k = 0; k < W; ++k) {
+                        const uint32_t e = e0 + 32 * k;
+                        if (e < both) {
+                            const unsigned long long d = e >= LE ? de[1] : de[0];
                             const bool h = HOT && (d & 1ull);
-                            const uint64_t off = (d >> 3) * 2 + c[k];
+                            const uint64_t off = (d >> 3) * 2 + (e >= LE ? e - LE : e);
                             E::reduce(h ? A.slab : A.table, off, a[k]);
                             if (TWO) E::reduce(h ? B.slab : B.table, off, b[k]);
                         }
                     }
-                }
+                };
+                if (!PARTS && LE <= PUSH_SHORT) turn(lane, std::integral_constant<int, 2>());
+                else for (uint32_t e0 = lane; e0 < both; e0 += 32 * PUSH_WIDE) turn(e0, std::integral_constant<int, PUSH_WIDE>());
                 continue;
             }
             for (uint32_t c = lane; c < LE; c += 32) {

@@ -46,3 +46,10 @@ def test_every_row_is_pulled_and_pushed_once(value_bytes, L, hot_n):
     for which in (0, 1):
         assert np.array_equal(s.read_table(which).cpu().numpy(), o.table(which))
     s.close()
+
+
+@pytest.mark.parametrize("hot_n", [0, 60])
+@pytest.mark.parametrize("L", [30, 32, 66, 128])
+def test_8_byte_rows_of_a_whole_turn_and_a_little_less_and_more(L, hot_n):
+    # a turn takes 128 values of two rows; 64 where rows have at most 32 and no warps share a window
+    test_every_row_is_pulled_and_pushed_once(8, L, hot_n)
