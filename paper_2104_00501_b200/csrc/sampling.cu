@@ -737,13 +737,16 @@ lt_walk_kernel(View v, HandleView h, uint64_t N, uint64_t cursor, uint64_t n, ui
 // instruction, as gather8_kernel does), which saves the separate gather launch of a PullSample with values.  The 32 entries
 // of a word are then shared by `sharers` warps (1, 2 or 4): all of them find out where the entries go, the first one writes
 // that down, and each copies its part of the rows.  A call on two sub-handles of 15,000 entries has 940 words, and one warp
-// per word waited for four rows at a time eight times over.  Measured: 21,756 samples in four parts 64.5 -> 49.5 us, 14,380
-// of 64 floats in one 21.3 -> 18.6 us.
-template <int C8>
+// per word waited for four rows at a time eight times over.  Measured: 21,756 samples of 128 floats in four parts 68.0 -> 50.1 us, 14,380
+// of 64 floats in one 21.8 -> 19.5 us.  UNR: instructions with rows in flight per warp.  Four take 64 registers, so 32 resident
+// warps per multiprocessor in place of 48, and pay where few rows are copied (128 floats: 400,000 samples in four parts 124.5 -> 105 us,
+// 1M in four 184 -> 176.5, 1M in 64 1,090 -> 1,020); two are better from where the rows fill more than two rounds of 32 warps
+// (400,000 at once 66.6 -> 64.1, 1M 134.2 -> 129.7; in between, 240,000 at once 50.1 -> 50.5).
+template <int C8, unsigned SHARERS, int UNR>
 __global__ void __launch_bounds__(256)
 lt_place_kernel(View v, HandleView h, uint64_t N, uint64_t cursor, uint64_t n, uint32_t q_first,
                 uint32_t* __restrict__ out, const float* __restrict__ table, const float* slab,
-                float* __restrict__ out_vals, unsigned sharers)
+                float* __restrict__ out_vals)
 {
     grid_dependency_wait();
     const LtChunk c = lt_chunk(q_first + blockIdx.y, N, v.R, cursor, n);
@@ -754,8 +757,8 @@ lt_place_kernel(View v, HandleView h, uint64_t N, uint64_t cursor, uint64_t n, u
     // the first warps take the words of the fresh entries that are walked, those after them the entries that earlier
     // calls postponed and this one emits (they come after the local ones)
     const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const uint64_t w = C8 > 0 ? warp / sharers : warp;
-    const unsigned share = C8 > 0 ? (unsigned)(warp % sharers) : 0u;
+    const uint64_t w = warp / SHARERS;
+    const unsigned share = (unsigned)(warp % SHARERS);
     const bool writes = share == 0;                                  // places are written down once
     const uint64_t words = wk.x ? ((end + 31) >> 5) - (oc >> 5) : 0;
     const uint64_t old = cnt < pt - ph ? cnt : pt - ph;
@@ -800,14 +803,15 @@ lt_place_kernel(View v, HandleView h, uint64_t N, uint64_t cursor, uint64_t n, u
     }
     if (writes) count_sample(v, key, emitted);
     if (C8 > 0) {
-        constexpr int RPI = C8 > 0 ? 32 / C8 : 1, UNR = RPI >= 4 ? 2 : 4;       // rows per instruction; instructions in flight
-        const int rows = 32 / (int)sharers, r_first = (int)share * rows;         // a multiple of the UNR * RPI rows of a turn
+        constexpr int RPI = C8 > 0 ? 32 / C8 : 1, ROWS = 32 / (int)SHARERS;      // rows per instruction; per warp
+        static_assert(ROWS % (UNR * RPI) == 0, "whole turns");
         const unsigned sub = lane / (C8 > 0 ? C8 : 1), ch = lane % (C8 > 0 ? C8 : 1);
         const uint64_t L = (uint64_t)v.L4 * 4;
         const uint32_t src = emitted ? key : 0xFFFFFFFFu;
         uint32_t pend = 0xFFFFFFFFu;                                 // replica row of a replicated key
         if (emitted && key_is_hot(v, key)) pend = c.q * (uint32_t)v.Hcap + (uint32_t)__ldg(v.slot_of + key);
-        for (int r0 = r_first; r0 < r_first + rows; r0 += UNR * RPI) {
+        for (int r1 = 0; r1 < ROWS; r1 += UNR * RPI) {
+            const int r0 = (int)share * ROWS + r1;
             uint32_t so[UNR], po[UNR], oo[UNR];
             F8 a[UNR];
 #pragma unroll
@@ -874,10 +878,16 @@ static nups_status pull_internal(nups_store* s, int id, uint64_t n, uint32_t* d_
         while (fused && sharers < 4 && (uint64_t)by_word.x * by_word.y * 8 * sharers * 2 <= (uint64_t)s->sm_count * 32) sharers *= 2;
         const dim3 shared_words(grid_for((max_size / 32 + 4) * sharers, 8), by_word.y);
         if (fused) nups_time_begin(s, st, NUPS_TIMED_SAMPLE_ROWS);
-        if (fused && c8 == 8) nups_launch_dependent(lt_place_kernel<8>, shared_words, 256, 0, st, v, hv, h.N, h.cursor, n, qf, d_keys_out, s->val, s->dval, d_vals_out, sharers);
-        else if (fused && c8 == 16) nups_launch_dependent(lt_place_kernel<16>, shared_words, 256, 0, st, v, hv, h.N, h.cursor, n, qf, d_keys_out, s->val, s->dval, d_vals_out, sharers);
-        else if (fused) nups_launch_dependent(lt_place_kernel<32>, shared_words, 256, 0, st, v, hv, h.N, h.cursor, n, qf, d_keys_out, s->val, s->dval, d_vals_out, sharers);
-        else nups_launch_dependent(lt_place_kernel<0>, by_word, 256, 0, st, v, hv, h.N, h.cursor, n, qf, d_keys_out, nullptr, nullptr, nullptr, 1u);
+        const bool deep = n <= (uint64_t)s->sm_count * 32 * 64;         // rows in two rounds of resident warps, see lt_place_kernel
+#define NUPS_PLACE(C8_, DEEP_)                                                                                            \
+    nups_launch_dependent(sharers == 4 ? lt_place_kernel<C8_, 4, DEEP_> : sharers == 2 ? lt_place_kernel<C8_, 2, DEEP_>   \
+                          : deep ? lt_place_kernel<C8_, 1, DEEP_> : lt_place_kernel<C8_, 1, 2>, shared_words, 256, 0, st, v, hv, h.N, \
+                          h.cursor, n, qf, d_keys_out, s->val, s->dval, d_vals_out)
+        if (fused && c8 == 8) NUPS_PLACE(8, 2);
+        else if (fused && c8 == 16) NUPS_PLACE(16, 4);
+        else if (fused) NUPS_PLACE(32, 4);
+#undef NUPS_PLACE
+        else nups_launch_dependent(lt_place_kernel<0, 1, 1>, by_word, 256, 0, st, v, hv, h.N, h.cursor, n, qf, d_keys_out, nullptr, nullptr, nullptr);
         if (fused) nups_time_end(s, st);
         LAUNCH_CHECK(s);
         if (fused) {

@@ -175,6 +175,41 @@ def test_full_pull_with_values_under_postponing_copies_the_rows_itself(L):
     assert np.array_equal(s.owner_of(dev_keys(allk)).cpu().numpy(), np.array([o.owner_of(k) for k in allk]))
 
 
+@pytest.mark.parametrize("L", [64, 128, 256])
+@pytest.mark.parametrize("per_warp,extra", [(12, 1), (40, -5), (64, 0), (64, 1)])
+def test_values_under_postponing_by_two_warps_and_by_one_per_word(per_warp, extra, L):
+    # samples per warp that is resident at 32 per multiprocessor: 32 entries are shared by four warps up to 8 samples, by two up to
+    # 16, then taken by one, which has fewer rows in flight from 64 on.  Whole handles and parts
+    resident = torch.cuda.get_device_properties(0).multi_processor_count * 32
+    nk, R, N = 5000, 16, per_warp * resident + extra
+    rng = np.random.default_rng(L + per_warp)
+    init = rng.normal(size=(nk, L)).astype(np.float32)
+    w = inputs.zipf_integer_weights(4000, 0.9).numpy().astype(np.uint32)
+    o, s = make_pair(nk, L, R=R, init=init, track_ownership=True)
+    hot = rng.choice(nk, 40, replace=False).astype(np.uint32)
+    o.set_management(hot, REPLICATE)
+    s.set_management(dev_keys(hot), REPLICATE)
+    d = rng.normal(size=(600, L)).astype(np.float32)
+    pk = rng.choice(hot, 600).astype(np.uint32)
+    o.push(pk, d)
+    s.push(dev_keys(pk), torch.from_numpy(d).cuda())
+    do = o.register_distribution(500, w, 4000, LONGTERM, U=4, G=50, seed=5)
+    ds = s.register_distribution(500, dev_keys(w), 4000, LONGTERM, U=4, G=50, seed=5)
+    for cuts in ([N], [N // 3 + 1, N // 2, N - N // 3 - 1 - N // 2]):
+        moved = rng.integers(0, nk, 3000).astype(np.uint32)
+        o.localize(moved)
+        s.localize(dev_keys(moved))
+        ho, hs = o.prepare_sample(do, N), s.prepare_sample(ds, N)
+        for c in cuts:
+            ko, vo = o.pull_sample(ho, c)
+            ks, vs = s.pull_sample(hs, c)
+            assert np.array_equal(host_keys(ks), ko)
+            assert torch.equal(vs.cpu(), torch.from_numpy(vo))
+    allk = np.arange(nk, dtype=np.uint32)
+    assert np.array_equal(s.owner_of(dev_keys(allk)).cpu().numpy(), np.array([o.owner_of(k) for k in allk]))
+    assert s.status_check() == 0
+
+
 @pytest.mark.parametrize("L,U,G,R", [(128, 16, 250, 8), (64, 4, 100, 3), (256, 16, 250, 8), (512, 3, 250, 2), (1024, 2, 40, 2)])
 def test_pooled_reuse_pull_sample_rows_are_what_each_worker_pulls(L, U, G, R):
     # The rows that PullSample returns are exactly what the sub-handle's worker pulls at that moment: the stored row
