@@ -289,6 +289,50 @@ def test_mf_by_column_over_several_windows_of_cells(per_warp, L, hot):
     assert s.status_check() == -4
 
 
+@pytest.mark.parametrize("clip", [0.0, 0.8])
+@pytest.mark.parametrize("per_warp,L", [(3, 100), (20, 100), (40, 8), (38, 200), (12, 300)])
+def test_mf_by_column_clips_counts_and_moves_as_the_oracle_does(per_warp, L, clip):
+    # two steps (the first one sets the bound of the second), nothing merged: the clipped updates and their statistics, access
+    # counts, owners, and what each worker's replicas hold.  Cells cannot race, as above; every third key is replicated
+    from oracle import Oracle
+    from paper_2104_00501_b200 import binding
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    n, R = sms * 5 * 4 * per_warp, 5
+    stretch, _ = _stretch_of_the_runs(n, L)
+    rng = np.random.default_rng(per_warp)
+    begins = (rng.random(n) < 0.2) | (np.arange(n) % stretch == 0)
+    M, N = n, int(begins.sum())
+    o = Oracle(M + N, L, workers=R, sync_interval=0, count_accesses=True, track_ownership=True)
+    s = binding.Store(M + N, L, workers=R, sync_interval=0, deterministic=False, clip_factor=clip, count_accesses=True, track_ownership=True)
+    o.set_clipping(clip)
+    o.init_uniform(0, 4, 0.3)
+    s.init_uniform(0, 4, 0.3)
+    hot = rng.permutation(M + N)[:(M + N) // 3].astype(np.uint32)
+    o.set_management(hot, REPLICATE)
+    s.set_management(dev_keys(hot), REPLICATE)
+    lb = loss_buf()
+    for _ in range(2):
+        i = rng.permutation(M).astype(np.uint32)
+        j = (M + rng.permutation(N)[np.cumsum(begins) - 1]).astype(np.uint32)
+        x = rng.normal(0, 1, n).astype(np.float32)
+        lo = o.step_mf(i, j, x, 0.01, 0.01)
+        s.step_mf(dev_keys(i), dev_keys(j), dev_f32(x), 0.01, 0.01, lb, by_column=True)
+        assert abs(lb.item() - lo) <= 1e-5 * abs(lo)
+    if clip:
+        (so, co), (ss, cs) = o.clip_stats(), s.clip_stats()
+        assert cs == co > 0 and ss == pytest.approx(so, rel=1e-5)
+    allk = np.arange(M + N, dtype=np.uint32)
+    assert np.array_equal(s.counts().cpu().numpy().astype(np.uint64), o.counts())
+    some = rng.choice(allk, 20_000, replace=False) if M + N > 20_000 else allk
+    assert np.array_equal(s.owner_of(dev_keys(some)).cpu().numpy(), np.array([o.owner_of(k) for k in some]))
+    keys = np.tile(hot[:2000], R)                                              # item block q of the pull belongs to worker q
+    np.testing.assert_allclose(s.pull(dev_keys(keys)).cpu().numpy(), o.pull(keys), rtol=RTOL, atol=ATOL)
+    o.sync()
+    s.sync()
+    np.testing.assert_allclose(s.read_table(0).cpu().numpy(), o.table(0), rtol=RTOL, atol=ATOL)
+    assert s.status_check() == 0
+
+
 @pytest.mark.parametrize("L", [8, 132])
 def test_mf_by_column_a_column_that_comes_back_shows_what_the_stretch_added_to_it(L):
     # a stretch of three windows: a first column, a second one to the window's end, a third for a window, the second one again.

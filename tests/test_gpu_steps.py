@@ -123,7 +123,7 @@ def test_mf_deterministic_parity(L, hot_n):
     assert np.array_equal(s.counts().cpu().numpy().astype(np.uint64), o.counts())
 
 
-@pytest.mark.parametrize("L,hot_n,n", [(100, 0, 4096), (100, 25, 4096), (8, 10, 3001), (300, 25, 1500)])
+@pytest.mark.parametrize("L,hot_n,n", [(100, 0, 4096), (100, 25, 4096), (8, 10, 3001), (300, 25, 1500), (300, 25, 6000)])
 def test_mf_fast_mode_on_cells_in_column_order(L, hot_n, n):
     # cells visited column by column (Section 5.1): fast mode sums a column's updates over a stretch of cells before
     # it adds them.  One step from the same start: every row's total update is the oracle's up to the races between
@@ -158,10 +158,11 @@ def test_mf_fast_mode_on_cells_in_column_order(L, hot_n, n):
     assert s.status_check() == 0
 
 
-def test_mf_by_column_takes_any_order_bad_keys_and_single_cells():
+@pytest.mark.parametrize("n", [701, 6007])          # below and above one cell per resident warp: the plain kernel and the one for runs
+def test_mf_by_column_takes_any_order_bad_keys_and_single_cells(n):
     # independent cells (hardly any runs), keys out of range in the middle and at the end, access counting and the
     # ownership map on: counts are exact, bad cells are skipped and flagged, every row's update is the oracle's
-    M, N, L, R, n = 60, 40, 100, 3, 701
+    M, N, L, R = 60, 40, 100, 3
     i, j, x = inputs.mf_cells(n, M, N, 0.8, 8, 0.1, 1)
     i, j, x = inputs.u32(i), inputs.u32(j), x.numpy()
     init = np.random.default_rng(1).normal(0, 0.3, size=(M + N, L)).astype(np.float32)
@@ -198,10 +199,11 @@ def test_mf_by_column_takes_any_order_bad_keys_and_single_cells():
     assert torch.equal(s.read_table(0), before)
 
 
-def test_mf_by_column_sends_each_cells_update_to_its_own_workers_replica():
+@pytest.mark.parametrize("n", [2003, 6007])
+def test_mf_by_column_sends_each_cells_update_to_its_own_workers_replica(n):
     # no merge after the step: a pull from worker q's part of a call sees the stored row plus q's pending updates
     # only, so the replicas must hold exactly the updates of the cells that belong to each worker
-    M, N, L, R, n = 80, 30, 100, 5, 2003
+    M, N, L, R = 80, 30, 100, 5
     i, j, x = inputs.mf_cells(n, M, N, 0.8, 8, 0.1, 4, by_column_of=30 * n)
     i, j, x = inputs.u32(i), inputs.u32(j), x.numpy()
     init = np.random.default_rng(4).normal(0, 0.3, size=(M + N, L)).astype(np.float32)
@@ -464,8 +466,10 @@ def test_fast_mode_with_clipping_tracks_the_clipped_oracle():
 @pytest.mark.parametrize("runs", [False, True])
 @pytest.mark.parametrize("n,L", [(2960, 100), (2961, 100), (7003, 200), (24_001, 12), (9001, 512)])
 def test_mf_by_column_with_bad_keys_at_the_sizes_where_its_batches_change(n, L, runs):
-    # a warp's stretch of 1, 2, 3, 9 (rounded to whole batches) and 4 cells, more than 32 with many cells; runs of one
-    # column and columns that change at every cell; keys out of range inside a batch: those cells change nothing
+    # 148 multiprocessors: one cell per resident warp (2,960, the plain kernel), then stretches of 2, 4, 12 (9 rounded to whole
+    # batches) and 4 cells; runs of one column and columns that change at every cell; keys out of range inside a batch: those
+    # cells change nothing.  Cells race here, so a lost update shows only where it is a good part of its row's; cells that
+    # cannot race, and stretches of several windows, are in test_gpu_fast_modes.py
     M, N, R = 3000, 900, 3
     i, j, x = inputs.mf_cells(n, M, N, 0.3, 8, 0.1, 2, by_column_of=20 * n if runs else 0)
     i, j, x = inputs.u32(i), inputs.u32(j), x.numpy()
@@ -478,9 +482,11 @@ def test_mf_by_column_with_bad_keys_at_the_sizes_where_its_batches_change(n, L, 
     lr = 2e-6                                  # tiny, see test_mf_fast_mode_on_cells_in_column_order
     bi = i.copy()
     bi[bad] = M + N + 7
-    s.step_mf(dev_keys(bi), dev_keys(j), dev_f32(x), lr, 0.01, loss_buf(), by_column=True)
+    lb = loss_buf()
+    s.step_mf(dev_keys(bi), dev_keys(j), dev_f32(x), lr, 0.01, lb, by_column=True)
     assert s.status_check() == -4
-    o.step_mf(bi, j, x, lr, 0.01)
+    lo = o.step_mf(bi, j, x, lr, 0.01)
+    assert abs(lb.item() - lo) <= 2e-3 * abs(lo)
     o.sync()
     s.sync()
     d_o = o.table(0).astype(np.float64) - init
