@@ -306,8 +306,12 @@ nups_status nups_step_mf(nups_store* store, const uint32_t* d_row, const uint32_
  * stretch of consecutive cells of that column that one warp works on (all cells
  * of such a stretch see the column's row from before the stretch, which is the
  * batch semantics of the deterministic mode).  Any order of cells gives a correct
- * step; the order only decides how much is saved.  In deterministic mode the
- * call is nups_step_mf.  Arguments, ownership and errors as nups_step_mf.      */
+ * step; the order only decides how much is saved.  Rows of row keys may be read
+ * up to seven cells of the stretch before they are used (their replicas up to
+ * three), so a row key that comes again within them may miss its last update.
+ * The call is nups_step_mf in deterministic mode and for batches of at most one
+ * cell per resident warp (20 per multiprocessor: 2,960 on 148), where there are
+ * no stretches to save on.  Arguments, ownership and errors as nups_step_mf.   */
 nups_status nups_step_mf_by_column(nups_store* store, const uint32_t* d_row, const uint32_t* d_col, const float* d_x,
                                    uint64_t n, float lr, float l2, float* d_loss_out, void* stream);
 

@@ -1414,13 +1414,17 @@ extern "C" nups_status nups_step_complex(nups_store* s, const uint32_t* d_h, con
 // replicated rows, of row and column keys, when the batch begins.  Columns that change inside a batch, keys out of range
 // between others and clipped updates take the cells of the batch one by one.
 // Bound by instruction issue and the latency of a warp's few cells: one cell at a time, with shuffled addresses and a
-// reduction of its own, took ~300 warp instructions.  65,536 cells: 100 floats 31.4 -> 20.3 us, 32 floats 27.2 -> 15.2;
-// 20,000 cells of 300 floats 40.1 -> 30.6.  What other cells see of one another's updates moves the step's loss: against one
-// cell at a time, by 1.2e-5 of it at 65,536 cells of 100 floats and 6.5e-5 at 20,000 (2.3e-5 and 1.1e-4 when the pending updates
-// were read a batch ahead, which was no faster for rows of at most 256 floats and 4 to 6 % faster for longer ones; 4.5e-4 when
-// they were read once per stretch, 18.7 us).
+// reduction of its own, took ~300 warp instructions.  65,536 cells (11M keys, rows not in cache): 100 floats 31.4 -> 21.4 us;
+// 2.2M keys: 32 floats 27.1 -> 15.0, 300 floats 112 -> 79; 20,000 cells of 300 floats 39.3 -> 30.3.
+// What cells see of one another's updates moves the step's loss: against one cell at a time, by 1.2e-5 of it at 65,536 cells of
+// 100 floats and 6.5e-5 at 20,000.  Pending updates read a batch ahead: 20.2 us, 2.3e-5 and 1.1e-4, and a warp does not see its own
+// updates of the batch before; read once per stretch: 18.7 us, 4.5e-4.
 // ---------------------------------------------------------------------------------------------
-constexpr int MF_RUN_BLOCKS = 5;          // resident blocks per multiprocessor the grid is sized for
+// Resident blocks per multiprocessor that the grid is sized for.  Five (96 registers) were measured best when a warp took one cell at a
+// time.  As the kernel is they make it spill wherever keys are replicated (228 bytes for rows of up to 128 floats, 1,956 for 512), and
+// fewer blocks are faster except without replicas: five / four / three 16.2 / 14.8 / 18.0 us for 65,536 cells of 100 floats, 8.1 / 7.2 /
+// 6.9 for 12,000, 78.9 / 39.7 / 36.9 for 65,536 of 300, 16.3 / 16.8 / 17.6 for 65,536 of 100 with nothing replicated.
+constexpr int MF_RUN_BLOCKS = 5;
 
 struct MfRows { const float4* read; float4* add; };       // the stored row; the row that takes the update (nullptr: no cell)
 
@@ -1445,7 +1449,9 @@ mf_runs_kernel(View v, const uint32_t* __restrict__ rowk, const uint32_t* __rest
     const float bound = CLIP ? clip_bound(v) : 0.f;
     float my_clip = 0.f;
     unsigned my_clipped = 0;
-    // whole batches, unless that would leave warps without a cell in a small call
+    // Whole batches once a warp has more than one.  Rounding up leaves warps idle: 11,840 cells are 4 per warp, 11,841 are 8 for
+    // half of the warps (7.3 and 7.8 us), 23,681 are 12 for two thirds (8.8 us at 23,680, 10.6); those calls are still faster than
+    // one cell at a time on all warps was (9.2 and 13.3 us).
     const uint64_t even = (n + nwarps - 1) / nwarps, stretch = even > B ? (even + B - 1) / B * B : even;
     const uint64_t first = warp * stretch < n ? warp * stretch : n;
     const uint64_t last = first + stretch < n ? first + stretch : n;            // this warp's cells: [first, last)
@@ -1795,8 +1801,10 @@ static nups_status mf_step(nups_store* s, const uint32_t* d_row, const uint32_t*
     rc = step_buffers(s, n, 2, false, &b);
     if (rc != NUPS_OK) return rc;
     View v = nups_view(s);
-    // The ordered mode is the same for any order.  A call with a cell per resident warp at most has no runs to save on, and the
-    // plain kernel has less to set up: 1,935 cells of 64 floats 5.9 us, 6.6 with the kernel for runs (65,536 cells: 102 and 20).
+    // The ordered mode is the same for any order.  With at most one cell per resident warp there are no runs to save on, and the
+    // plain kernel has less to set up: plain / runs 5.3 / 6.7 us for 1,935 cells of 64 floats, 6.9 / 7.5 for 2,960, 6.7 / 7.3 of
+    // 100 floats, 15.8 / 16.7 of 300.  From two cells per warp on the runs pay: 6.8 / 5.9 us for 2,961 cells of 64 floats,
+    // 7.0 / 5.9 of 100, 15.8 / 12.0 of 300, 10.1 / 6.8 for 6,000 of 100.
     const bool by_column = cells_by_column && !s->cfg.deterministic && n > (uint64_t)s->sm_count * MF_RUN_BLOCKS * 4;
     nups_time_begin(s, st, NUPS_TIMED_STEP);
     if (s->vb == 8) {

@@ -693,8 +693,8 @@ struct PushElement<true> {
 // keys show up early and often, so they take most accumulators, and a skewed batch stops queueing at a few L2
 // addresses even when its frequent keys were never marked for replication.
 // PARTS = several warps share a window of rows (see window_parts).  Calls that do not divide their windows do without its
-// registers: 400,000 rows of 128 floats pulled and pushed to two tables, no key replicated, 356 us with it (it spills) and 350
-// without; 300,000 rows of 128 8-byte values pushed 149.3 and 148.3 us.
+// registers: 400,000 rows of 128 floats pulled and pushed to two tables, no key replicated, 292 us with it (it spills) and 287
+// without; 300,000 rows of 128 8-byte values pushed 151.2 and 150.3 us (neither spills).
 template <bool HOT, bool TWO, int TIER, bool F64, bool PARTS>
 __global__ void __launch_bounds__(PUSH_THREADS, TWO ? PUSH_BLOCKS - 1 : PUSH_BLOCKS)
 push_atomic_kernel(View v, const uint32_t* __restrict__ keys, uint64_t n, PushPair A, PushPair B, uint64_t n_items,
@@ -1245,10 +1245,11 @@ push_chain_kernel(View v, const K* __restrict__ dest, const uint32_t* __restrict
 // Few rows: every block works out all rows' destinations (into shared memory), a warp per row looks whether an earlier row
 // has the same destination and, if none has, finds the later ones by scanning, 128 rows at a step, and adds them in order;
 // the first of its rows and the stored row move towards L2 meanwhile.
-// One launch in place of seven; the scans grow with n^2.  Measured: 100 rows 15 us (72 us before), 3,000 rows of 64 floats pushed
-// and merged 22.9 us (29.2 with scans of 32 rows and nothing asked for ahead), 3,000 rows of 64 floats alone, before that,
-// 28 us, while the sort and what follows it take 37 us for 4,500 rows, and a frequent key's chain is slower here (2,500
-// rows, a third of them of one key: 73 us): the line lies at 3,072.
+// One launch in place of seven; the scans grow with n^2.  Measured with the merge: 100 rows 7.2 us, 3,000 rows of 64 floats 18.3 to
+// 24.1 us by their skew (23.5 to 30.4 with scans of 32 rows and nothing asked for ahead).  The line lies below where any skew
+// makes the sort and what follows it the faster way: this kernel / the sort take, for uniform keys and for Zipf 1.4 with 1,000 keys
+// replicated, 18.3 / 28.8 and 24.6 / 33.0 us at 3,072 rows of 64 floats, 20.2 / 30.9 and 31.2 / 36.3 of 256 floats; at 4,096 rows
+// 22.2 / 29.4 and 34.2 / 33.4, 24.4 / 32.1 and 44.9 / 37.7; at 5,000 30.6 / 30.4 and 40.6 / 34.8, 33.2 / 33.2 and 53.6 / 39.5.
 constexpr uint32_t SMALL_PUSH_ROWS = 3072;
 constexpr unsigned SMALL_THREADS = 256, SMALL_LIST = 512;
 static_assert(SMALL_PUSH_ROWS <= 65536, "row numbers are kept in 16 bits");
